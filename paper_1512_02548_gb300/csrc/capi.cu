@@ -159,7 +159,7 @@ struct sem_mesh {
   SolveRecord* rec = nullptr;
   // workspace
   double *Phi = nullptr, *qtmp = nullptr, *edgetmp = nullptr;
-  double *wt = nullptr, *etax = nullptr, *phisx = nullptr, *R = nullptr, *scr = nullptr;
+  double *wt = nullptr, *etax = nullptr, *phisx = nullptr, *R = nullptr, *R2 = nullptr, *ub = nullptr;
   double *ke = nullptr, *kp = nullptr, *ae = nullptr, *ap = nullptr, *se = nullptr, *sp = nullptr;
   double *eta_dev = nullptr, *phis_dev = nullptr;
   double *s1e = nullptr, *s1p = nullptr;   // second stage-input pair of the fused RK stage
@@ -305,11 +305,9 @@ int do_rhs(sem_mesh* m, const double* eta, const double* phis, double time, doub
   if (rc0) return rc0;
   int rc = do_solve(m, phis, m->Phi, s);
   if (rc) return rc;
-  CUDA_TRY(launch_wsurf(m->st, m->Phi, eta, m->wt, s));
-  CUDA_TRY(launch_sx(m->st, eta, phis, m->R, s));
-  CUDA_TRY(launch_mass1d(m->st, m->R, 2, m->etax, m->phisx, m->scr, s));
+  CUDA_TRY(launch_recover(m->st, m->Phi, eta, phis, m->wt, m->etax, m->phisx, s));
   CUDA_TRY(launch_zakharov(m->st, eta, m->etax, m->phisx, m->wt, m->R, s));
-  CUDA_TRY(launch_mass1d(m->st, m->R, 2, de, dp, m->scr, s));
+  CUDA_TRY(launch_mass1d(m->st, m->R, de, dp, s));
   if (has_zones(m)) CUDA_TRY(launch_relax(m->st, eta, phis, time, 1.0 / tau, de, dp, s));
   (void)Q;
   return SEM_OK;
@@ -340,7 +338,7 @@ Instance make_instance(sem_mesh* m, double* eta, double* phis, double tstart, do
   I.eta = eta; I.phis = phis;
   I.s0e = m->se; I.s0p = m->sp; I.s1e = m->s1e; I.s1p = m->s1p;
   I.ke = m->ke; I.kp = m->kp; I.ae = m->ae; I.ap = m->ap;
-  I.wt = m->wt; I.etax = m->etax; I.phisx = m->phisx; I.R = m->R; I.scr = m->scr;
+  I.wt = m->wt; I.R = m->R; I.R2 = m->R2; I.ub = m->ub; I.ub_stride = m->p.Nx + m->grid + 1;
   I.P1 = m->Phi1; I.P2 = m->Phi2; I.P3 = m->Phi3; I.D32 = m->D32;
   I.hist = (m->hist_dt == dt && m->hist_eta == eta && m->hist_phis == phis) ? 1 : 0;
   I.tstart = tstart; I.dt = dt;
@@ -396,17 +394,6 @@ int do_rk4(sem_mesh* m, double* eta, double* phis, double t0, double dt, int nst
   return SEM_OK;
 }
 
-std::vector<double> matmul(const std::vector<double>& A, const std::vector<double>& B, int n, int k, int mcols) {
-  std::vector<double> C((size_t)n * mcols, 0.0);
-  for (int i = 0; i < n; ++i)
-    for (int j = 0; j < mcols; ++j) {
-      long double s = 0.0L;
-      for (int q = 0; q < k; ++q) s += (long double)A[(size_t)i * k + q] * B[(size_t)q * mcols + j];
-      C[(size_t)i * mcols + j] = (double)s;
-    }
-  return C;
-}
-
 }  // namespace
 
 extern "C" {
@@ -418,7 +405,8 @@ int64_t sem_launch_count(void) { return g_launches.load(); }
 // Host tables of one (P, Nz, Pf, filter) combination, shared by every mesh that has it.
 struct ColumnTables {
   Line L;
-  std::vector<double> MD, I, B, F, wrow, Aii, Z, Sg, lam, dsl, sig;
+  std::vector<double> SX, I, ZB, F, wrow, Z, Sg, lam, dsl, sig;
+  int win = 0;
   long double S00 = 0, S01 = 0, S11 = 0;
 };
 
@@ -451,11 +439,7 @@ static int column_tables(const sem_params& p, std::shared_ptr<const ColumnTables
     t->sig[iz] = (double)l / Nz + 0.5 * (L.r[b] + 1.0) * dsl[l];
   }
   t->sig[nrow - 1] = 1.0;
-  t->MD = matmul(L.M, L.D, Q, Q, Q);
   t->I = interpolation(L, Lf);                                        // Qf×Q
-  std::vector<double> It(Q * Qf);
-  for (int q = 0; q < Qf; ++q) for (int c = 0; c < Q; ++c) It[c * Qf + q] = t->I[q * Q + c];
-  t->B = matmul(It, Lf.M, Q, Qf, Qf);                                 // Q×Qf = Iᵀ M_f
   t->F = filter_matrix(L, p.filter_alpha, p.filter_s, p.filter_ic);
   // w̃ weights: v = M_σ⁻¹ e_top, c_l = (Δσ_l/2) M v|_l, contracted with the layer's σ-derivative
   // (2/Δσ_l) D into one weight per row: w̃ d = Σ_iz wrow_iz Φ_iz
@@ -475,14 +459,14 @@ static int column_tables(const sem_params& p, std::shared_ptr<const ColumnTables
       }
     for (int iz = 0; iz < nrow; ++iz) t->wrow[iz] = (double)wr[iz];
   }
-  // static condensation of M' (element scale Δx/2 · M)
-  t->Aii.assign((size_t)Pm * Pm, 0.0);
+  // static condensation of M' (element scale Δx/2 · M): Z = M_bi M_ii⁻¹, the Schur complement, and the
+  // element right-hand sides R = T f (T = M·D, Iᵀ M_f) condensed: boundary rows T_b − Z T_i, interior
+  // rows M_ii⁻¹ T_i
   t->Z.assign((size_t)2 * Pm, 0.0);
   {
     std::vector<long double> Mii((size_t)Pm * Pm);
     for (int i = 0; i < Pm; ++i) for (int k = 0; k < Pm; ++k) Mii[i * Pm + k] = L.M[(i + 1) * Q + (k + 1)];
     if (!invert(Mii, Pm)) return fail(SEM_ERR_INVALID_ARG, "interior mass is singular");
-    for (int i = 0; i < Pm * Pm; ++i) t->Aii[i] = (double)Mii[i];
     const int bn[2] = {0, P};
     long double Zl[2][kMaxP];
     for (int s2 = 0; s2 < 2; ++s2)
@@ -498,6 +482,33 @@ static int column_tables(const sem_params& p, std::shared_ptr<const ColumnTables
       return acc;
     };
     t->S00 = sch(0, 0); t->S01 = sch(0, 1); t->S11 = sch(1, 1);
+    auto condensed = [&](const std::vector<double>& Lf_, const std::vector<double>& Rt, int k, int nc) {
+      // T = Lf_ (Q×k) · Rt (k×nc) in long double, then its condensed rows
+      std::vector<long double> T((size_t)Q * nc, 0.0L);
+      for (int a = 0; a < Q; ++a)
+        for (int c = 0; c < nc; ++c)
+          for (int q = 0; q < k; ++q) T[(size_t)a * nc + c] += (long double)Lf_[(size_t)a * k + q] * Rt[(size_t)q * nc + c];
+      std::vector<double> out((size_t)Q * nc);
+      for (int c = 0; c < nc; ++c) {
+        long double b0 = T[c], b1 = T[(size_t)P * nc + c];
+        for (int i = 0; i < Pm; ++i) {
+          b0 -= Zl[0][i] * T[(size_t)(1 + i) * nc + c];
+          b1 -= Zl[1][i] * T[(size_t)(1 + i) * nc + c];
+          long double v = 0.0L;
+          for (int m2 = 0; m2 < Pm; ++m2) v += Mii[i * Pm + m2] * T[(size_t)(1 + m2) * nc + c];
+          out[(size_t)(1 + i) * nc + c] = (double)v;
+        }
+        out[c] = (double)b0;
+        out[(size_t)P * nc + c] = (double)b1;
+      }
+      return out;
+    };
+    std::vector<double> It((size_t)Q * Qf);
+    for (int q = 0; q < Qf; ++q) for (int c = 0; c < Q; ++c) It[(size_t)c * Qf + q] = t->I[(size_t)q * Q + c];
+    t->SX = condensed(L.M, L.D, Q, Q);
+    t->ZB = condensed(It, Lf.M, Qf, Qf);
+    // |S01|/S00 = 1/(P+1) bounds the decay of the interface factors (surface_device.cuh)
+    t->win = (int)std::ceil(18.0L * std::log(10.0L) / std::log(t->S00 / std::fabs(t->S01)));
   }
   // σ-separable preconditioner: Kσ S = Mσ S Λ on the interior rows (Dirichlet at the surface),
   // Kσ = Σ_l (2/Δσ_l) Dᵀ W D, Mσ = Σ_l (Δσ_l/2) W (GLL-lumped, as in the stiffness quadrature).
@@ -588,12 +599,9 @@ static int mesh_create_impl(const sem_params* pin, const double* x_edges_h, cons
   rc = column_tables(p, &ct);
   if (rc) return rc;
   const Line& L = ct->L;
-  const std::vector<double>& MD = ct->MD;
   const std::vector<double>& I = ct->I;
-  const std::vector<double>& B = ct->B;
   const std::vector<double>& F = ct->F;
   const std::vector<double>& wrow = ct->wrow;
-  const std::vector<double>& Aii = ct->Aii;
   const std::vector<double>& Z = ct->Z;
   const std::vector<double>& Sg = ct->Sg;
   const std::vector<double>& lam = ct->lam;
@@ -611,10 +619,10 @@ static int mesh_create_impl(const sem_params* pin, const double* x_edges_h, cons
       }
       hx_loc[(size_t)e * Q + a] = s * 2.0 / dxe[e];
     }
-  // M' interface tridiagonal (Thomas factors; Sherman–Morrison closure when periodic)
+  // M' interface tridiagonal: pivots p_j = d_j − e²_{j−1}/p_{j−1}, around the ring until they repeat when
+  // periodic (the factors of a cyclic bidiagonal LDLᵀ; their start is forgotten within ct->win steps)
   const int N = p.periodic ? Nx : Nx + 1;
-  std::vector<double> th_e(N, 0.0), th_m(N, 0.0), th_cp(N, 0.0), th_z(N, 0.0);
-  double th_vlast = 0.0, th_fac = 0.0;
+  std::vector<double> th_al(N, 0.0), th_m(N, 0.0), th_cp(N, 0.0);
   {
     const double S00 = ct->S00, S01 = ct->S01, S11 = ct->S11;
     std::vector<double> d(N, 0.0), e(N, 0.0);
@@ -622,32 +630,19 @@ static int mesh_create_impl(const sem_params* pin, const double* x_edges_h, cons
       const int jr = (j + 1) % N;
       d[j] += se[j] * S00;
       d[jr] += se[j] * S11;
-      e[j] = se[j] * S01;            // coupling j ↔ j+1 (periodic: e[N−1] is the corner)
+      e[j] = se[j] * S01;            // coupling j ↔ j+1 (periodic: e[N−1] couples N−1 and 0)
     }
-    double gamma = 0.0, corner = 0.0;
-    if (p.periodic) {
-      corner = e[N - 1];
-      gamma = -d[0];
-      d[0] -= gamma;
-      d[N - 1] -= corner * corner / gamma;
-    }
-    std::vector<double> m(N), cp(N, 0.0);
+    double l = 0.0;                  // multiplier e_{j−1}/p_{j−1}
+    if (p.periodic)
+      for (int k = ct->win; k > 0; --k) {
+        const int j = ((N - k) % N + N) % N;
+        l = e[j] / (d[j] - e[(j + N - 1) % N] * l);
+      }
     for (int j = 0; j < N; ++j) {
-      const double piv = j == 0 ? d[0] : d[j] - e[j - 1] * cp[j - 1];
-      m[j] = 1.0 / piv;
-      if (j < N - 1) cp[j] = e[j] * m[j];
-    }
-    th_e = e; th_m = m; th_cp = cp;
-    if (p.periodic) {
-      std::vector<double> u(N, 0.0), y(N);
-      u[0] = gamma;
-      u[N - 1] = corner;
-      for (int j = 0; j < N; ++j) y[j] = (j == 0 ? u[0] : u[j] - e[j - 1] * y[j - 1]) * m[j];
-      for (int j = N - 2; j >= 0; --j) y[j] -= cp[j] * y[j + 1];
-      const double vl = corner / gamma;
-      th_z = y;
-      th_vlast = vl;
-      th_fac = 1.0 / (1.0 + y[0] + vl * y[N - 1]);
+      const double ep = j > 0 ? e[j - 1] : (p.periodic ? e[N - 1] : 0.0);
+      th_m[j] = 1.0 / (d[j] - ep * l);
+      th_al[j] = -ep * th_m[j];
+      l = th_cp[j] = e[j] * th_m[j];
     }
   }
   const int nr = nrow - 1;
@@ -672,11 +667,10 @@ static int mesh_create_impl(const sem_params* pin, const double* x_edges_h, cons
   const size_t o_S32 = cv.take<float>((size_t)nr * nr), o_ST32 = cv.take<float>((size_t)nr * nr),
                o_lam = cv.take<double>(nr), o_xcol = cv.take<double>(ncol);
   // surface tables
-  const size_t o_tD = cv.take<double>(Q * Q), o_tMD = cv.take<double>(Q * Q), o_tB = cv.take<double>((size_t)Q * Qf),
+  const size_t o_tD = cv.take<double>(Q * Q), o_tSX = cv.take<double>(Q * Q), o_tZB = cv.take<double>((size_t)Q * Qf),
                o_tI = cv.take<double>((size_t)Qf * Q), o_tF = cv.take<double>(Q * Q), o_twr = cv.take<double>((size_t)nrow),
-               o_tAii = cv.take<double>((size_t)Pm * Pm + 1), o_tZ = cv.take<double>((size_t)2 * Pm + 1),
-               o_tse = cv.take<double>(Nx), o_te = cv.take<double>(N), o_tm = cv.take<double>(N),
-               o_tcp = cv.take<double>(N), o_tz = cv.take<double>(N);
+               o_tZ = cv.take<double>((size_t)2 * Pm + 1), o_tse = cv.take<double>(Nx), o_tal = cv.take<double>(N),
+               o_tm = cv.take<double>(N), o_tcp = cv.take<double>(N);
   const size_t up_end = cv.off;
   const size_t o_geo64 = cv.take<double>((size_t)Nx * Q * 4),
                o_geo32 = cv.take<float>((size_t)Nx * Q * 4), o_id64 = cv.take<double>(n), o_id32 = cv.take<float>(n),
@@ -704,7 +698,8 @@ static int mesh_create_impl(const sem_params* pin, const double* x_edges_h, cons
   const bool zones = p.relax_left > 0.0 || p.relax_right > 0.0;
   const size_t o_wA = cv.take<double>(zones ? 4 * kMaxWaveComp : 0), o_wEP = cv.take<double>(zones ? 2 * ncol : 0);
   const size_t o_wt = cv.take<double>(ncol), o_etax = cv.take<double>(ncol), o_phisx = cv.take<double>(ncol),
-               o_R = cv.take<double>((size_t)2 * Nx * Q), o_scr = cv.take<double>((size_t)4 * Nx + 2 * (N + 1)),
+               o_R = cv.take<double>((size_t)2 * Nx * Q), o_R2 = cv.take<double>((size_t)2 * Nx * Q),
+               o_ub = cv.take<double>((size_t)2 * (Nx + m->grid + 1)),
                o_ke = cv.take<double>(ncol), o_kp = cv.take<double>(ncol), o_ae = cv.take<double>(ncol),
                o_ap = cv.take<double>(ncol), o_se = cv.take<double>(ncol), o_sp = cv.take<double>(ncol),
                o_etad = cv.take<double>(ncol), o_phisd = cv.take<double>(ncol),
@@ -749,8 +744,8 @@ static int mesh_create_impl(const sem_params* pin, const double* x_edges_h, cons
     for (int e = 0; e < Nx; ++e) r2dx[e] = 2.0 / dxe[e];
     up(o_r2dx, r2dx);
   }
-  up(o_tD, L.D); up(o_tMD, MD); up(o_tB, B); up(o_tI, I); up(o_tF, F); up(o_twr, wrow);
-  up(o_tAii, Aii); up(o_tZ, Z); up(o_tse, se); up(o_te, th_e); up(o_tm, th_m); up(o_tcp, th_cp); up(o_tz, th_z);
+  up(o_tD, L.D); up(o_tSX, ct->SX); up(o_tZB, ct->ZB); up(o_tI, I); up(o_tF, F); up(o_twr, wrow);
+  up(o_tZ, Z); up(o_tse, se); up(o_tal, th_al); up(o_tm, th_m); up(o_tcp, th_cp);
   up(o_lam, lam);
   {
     std::vector<double> xc(ncol);
@@ -818,7 +813,7 @@ static int mesh_create_impl(const sem_params* pin, const double* x_edges_h, cons
   a.pv32 = ps.v32;
 
   m->Phi = D_(o_Phi); m->qtmp = D_(o_qtmp); m->edgetmp = D_(o_etmp);
-  m->wt = D_(o_wt); m->etax = D_(o_etax); m->phisx = D_(o_phisx); m->R = D_(o_R); m->scr = D_(o_scr);
+  m->wt = D_(o_wt); m->etax = D_(o_etax); m->phisx = D_(o_phisx); m->R = D_(o_R); m->R2 = D_(o_R2); m->ub = D_(o_ub);
   m->ke = D_(o_ke); m->kp = D_(o_kp); m->ae = D_(o_ae); m->ap = D_(o_ap); m->se = D_(o_se); m->sp = D_(o_sp);
   m->eta_dev = D_(o_etad); m->phis_dev = D_(o_phisd);
   m->s1e = D_(o_s1e); m->s1p = D_(o_s1p);
@@ -829,10 +824,9 @@ static int mesh_create_impl(const sem_params* pin, const double* x_edges_h, cons
 
   SurfTables& t = m->st;
   t.P = P; t.Pf = p.Pf; t.Nx = Nx; t.Nz = Nz; t.ncol = ncol; t.nrow = nrow; t.periodic = g.periodic; t.g = p.g;
-  t.D = D_(o_tD); t.MD = D_(o_tMD); t.B = D_(o_tB); t.I = D_(o_tI); t.F = D_(o_tF); t.wrow = D_(o_twr);
-  t.Aii = D_(o_tAii); t.Z = D_(o_tZ); t.se = D_(o_tse); t.dsl = g.dsl; t.h = g.h;
-  t.th_e = D_(o_te); t.th_m = D_(o_tm); t.th_cp = D_(o_tcp); t.th_z = D_(o_tz);
-  t.th_vlast = th_vlast; t.th_fac = th_fac; t.nif = N; t.filter_on = (p.filter_ic >= 0 && p.filter_ic < P) ? 1 : 0;
+  t.D = D_(o_tD); t.SX = D_(o_tSX); t.ZB = D_(o_tZB); t.I = D_(o_tI); t.F = D_(o_tF); t.wrow = D_(o_twr);
+  t.Z = D_(o_tZ); t.se = D_(o_tse); t.r2dx = g.r2dx; t.dsl = g.dsl; t.h = g.h;
+  t.th_al = D_(o_tal); t.th_m = D_(o_tm); t.th_cp = D_(o_tcp); t.win = ct->win; t.nif = N; t.filter_on = (p.filter_ic >= 0 && p.filter_ic < P) ? 1 : 0;
   t.xcol = D_(o_xcol); t.x0 = x_edges_h[0]; t.x1 = x_edges_h[Nx];
   t.relax_left = p.relax_left; t.relax_right = p.relax_right; t.ncomp = 0; t.wave = D_(o_wave);
   t.nzl = 0; t.wkx = nullptr;
@@ -985,9 +979,7 @@ int sem_recover_gradient(sem_mesh* m, const double* Phi_d, const double* eta_d, 
     return fail(SEM_ERR_INVALID_ARG, "NULL argument");
   DeviceGuard dg(m->device);
   cudaStream_t s = (cudaStream_t)stream;
-  CUDA_TRY(launch_wsurf(m->st, Phi_d, eta_d, w_surf_d, s));
-  CUDA_TRY(launch_sx(m->st, eta_d, phis_d, m->R, s));
-  CUDA_TRY(launch_mass1d(m->st, m->R, 2, etax_d, phisx_d, m->scr, s));
+  CUDA_TRY(launch_recover(m->st, Phi_d, eta_d, phis_d, w_surf_d, etax_d, phisx_d, s));
   return SEM_OK;
 }
 

@@ -6,43 +6,86 @@
 //        w̃(x_i) = Σ_l Σ_b c_{l,b} · (1/d_i) (2/Δσ_l) (D Φ_{i,l})_b,
 //    with c_l = (Δσ_l/2) M · (M_σ⁻¹ e_top)|_layer l precomputed on the host.  No 2D mass
 //    solve is needed; the result equals the global projection up to rounding.
-//  * S_x f and the over-integrated Zakharov integrals are formed per element
-//    (unassembled), and one kernel solves M' u = Σ_e Q_eᵀ R_e by static condensation:
-//    element-interior unknowns are eliminated with the precomputed M_ii⁻¹, the interface
-//    unknowns form a tridiagonal system (cyclic when periodic, closed by
-//    Sherman–Morrison) solved with precomputed Thomas factors, then the interiors are
-//    recovered.  M' is constant in time, so only the right-hand sides change.
+//  * M' u = Σ_e Q_eᵀ R_e is solved by static condensation: the element interiors are
+//    eliminated in the host tables (S_x f and the over-integrated Zakharov integrals are
+//    formed condensed), the interface unknowns form a tridiagonal system (cyclic when
+//    periodic) whose factors decay, so each block solves for its own elements from a
+//    window of their neighbours (surface_device.cuh).
 //  * The modal filter F = V̂SV̂⁻¹ acts per element on interior nodes only: the hat
 //    modes are untouched, so shared end values are unchanged by construction.
 #include "surface_device.cuh"
 
 namespace semgb {
 
-__global__ void k_wsurf(SurfTables t, const double* __restrict__ Phi, const double* __restrict__ eta,
-                        double* __restrict__ w) {
-  const int col = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (col >= t.ncol) return;
-  wsurf_column(t, Phi, eta, w, col, threadIdx.x & 31);
+// The M' solves run per block of kRecElems elements: the block's window of condensed right-hand sides
+// (its own elements and t.win + 1 more on either side) is enough for its interface unknowns
+// (mass1d_window), so no block waits for another.
+constexpr int kRecElems = 16, kRecThreads = 128;
+
+// Gradient recovery: w̃ of the block's columns, S_x of η and φ̃ (boundary rows for the whole window, kept in
+// shared memory), the interface solves and the block's columns of ∂xη and ∂xφ̃.  Latency bound: one
+// launch of Nx/16 blocks instead of three launches, the last of which solved the whole chain on one
+// SM.  1001×2, P = 6, with two filter calls and their copies: 148 → 51 µs, now the host's calls.
+__global__ void __launch_bounds__(kRecThreads) k_recover(SurfTables t, const double* __restrict__ Phi,
+                                                         const double* __restrict__ eta,
+                                                         const double* __restrict__ phis, double* __restrict__ w,
+                                                         double* __restrict__ etax, double* __restrict__ phisx) {
+  extern __shared__ double sm[];
+  const int Nx = t.Nx, P = t.P, N = t.nif, W = t.win;
+  const int e0 = blockIdx.x * kRecElems, e1 = min(Nx, e0 + kRecElems), ne = e1 - e0;
+  const int nwin = ne + 2 * W + 2;                    // elements e0 − W − 1 … e1 + W
+  double* gl = sm;                                    // [2][nwin] left and right boundary rows
+  double* gr = gl + 2 * nwin;
+  double* ub = gr + 2 * nwin;                         // [2][kRecElems + 1]
+  for (int k = threadIdx.x; k < 4 * nwin; k += blockDim.x) {
+    const int i = k >> 2, fld = (k >> 1) & 1, end = k & 1;
+    int ex = e0 - W - 1 + i;
+    if (t.periodic) { ex %= Nx; if (ex < 0) ex += Nx; }
+    const double v = (ex >= 0 && ex < Nx) ? sx_value(t, fld ? phis : eta, ex, end ? P : 0) : 0.0;
+    (end ? gr : gl)[fld * nwin + i] = v;
+  }
+  const int c0 = e0 * P, c1 = e1 * P + ((!t.periodic && e1 == Nx) ? 1 : 0);
+  for (int q0 = 0; q0 < 8 * (c1 - c0); q0 += blockDim.x) {
+    const int q = q0 + threadIdx.x, col = c0 + (q >> 3);
+    wsurf_column8(t, Phi, eta, w, col < c1 ? col : -1, q & 7);
+  }
+  __syncthreads();
+  const int rh = threadIdx.x >> 5;
+  if (rh < 2) {
+    // unknown j of the window sits between its elements i = j − (e0 − W − 1) − 1 and i
+    auto gfun = [&](int j) -> double {
+      int d = j - (e0 - W);                           // position in the window, around the ring
+      if (t.periodic) { d %= N; if (d < 0) d += N; }
+      return gl[rh * nwin + d + 1] + gr[rh * nwin + d];
+    };
+    mass1d_window(t, gfun, e0, ne + 1, [&](int i, double u) { ub[rh * (kRecElems + 1) + i] = u; });
+  }
+  __syncthreads();
+  for (int k = threadIdx.x; k < 2 * (c1 - c0); k += blockDim.x) {
+    const int fld = k >= c1 - c0 ? 1 : 0, col = c0 + k - fld * (c1 - c0);
+    const int i = min((col - c0) / P, ne - 1), a = col - c0 - i * P;
+    const double* u = ub + fld * (kRecElems + 1) + i;
+    double v = a == 0 ? u[0] : u[1];
+    if (a > 0 && a < P)
+      v = sx_value(t, fld ? phis : eta, e0 + i, a) - (t.Z[a - 1] * u[0] + t.Z[P - 1 + a - 1] * u[1]);
+    (fld ? phisx : etax)[col] = v;
+  }
 }
 
-__global__ void k_sx(SurfTables t, const double* __restrict__ f0, const double* __restrict__ f1,
-                     double* __restrict__ R) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= 2 * t.Nx * (t.P + 1)) return;
-  sx_item(t, f0, f1, R, k);
-}
-
-// One CTA: condensation, the interface solves (one warp per right-hand side), back-substitution.
-__global__ void k_mass1d(SurfTables t, const double* __restrict__ R, int nrhs, double* __restrict__ u0,
-                         double* __restrict__ u1, double* __restrict__ scr) {
-  for (int k = threadIdx.x; k < nrhs * t.Nx; k += blockDim.x) mass1d_condense(t, R, nrhs, scr, k);
+// M'u = Σ_e Q_eᵀ R_e from condensed right-hand sides, a block's columns from its own window.
+__global__ void __launch_bounds__(kRecThreads) k_mass1d(SurfTables t, const double* __restrict__ R,
+                                                        double* __restrict__ u0, double* __restrict__ u1) {
+  __shared__ double ub[2 * (kRecElems + 1)];
+  const int Nx = t.Nx, P = t.P, Q = P + 1;
+  const int e0 = blockIdx.x * kRecElems, e1 = min(Nx, e0 + kRecElems), ne = e1 - e0;
+  mass1d_windows(t, R, e0, e1, ub, kRecElems + 1);
   __syncthreads();
-  if ((threadIdx.x >> 5) < nrhs) mass1d_interface(t, nrhs, scr, threadIdx.x >> 5);
-  __syncthreads();
-  const int ncols = t.Nx * t.P + (t.periodic ? 0 : 1);
-  for (int k = threadIdx.x; k < nrhs * ncols; k += blockDim.x) {
-    const int rh = k / ncols, col = k - rh * ncols;
-    mass1d_backsub(t, R, nrhs, rh == 0 ? u0 : u1, scr, rh, col);
+  const int c0 = e0 * P, nc = ne * P + ((!t.periodic && e1 == Nx) ? 1 : 0);
+  for (int k = threadIdx.x; k < 2 * nc; k += blockDim.x) {
+    const int fld = k >= nc ? 1 : 0, c = k - fld * nc;
+    const int i = min(c / P, ne - 1);
+    const double* u = ub + fld * (kRecElems + 1) + i;
+    (fld ? u1 : u0)[c0 + c] = mass1d_value(t, R + ((size_t)fld * Nx + e0 + i) * Q, u[0], u[1], c - i * P);
   }
 }
 
@@ -53,15 +96,24 @@ __global__ void __launch_bounds__(32 * kZakWarps) k_zak(SurfTables t, const doub
                                                         const double* __restrict__ phisx,
                                                         const double* __restrict__ w,
                                                         double* __restrict__ R) {
-  __shared__ double sh[kZakWarps][kSurfWarpScratch];
-  const int wid = threadIdx.x >> 5;
-  const int ex = blockIdx.x * kZakWarps + wid;
-  if (ex >= t.Nx) return;
-  zak_element(t, eta, etax, phisx, w, R, ex, threadIdx.x & 31, sh[wid]);
+  __shared__ double sh[2 * kZakWarps][kSurfScratch];
+  const int half = threadIdx.x >> 4, sub = threadIdx.x & 15, Q = t.P + 1;
+  const int ex = blockIdx.x * 2 * kZakWarps + half;
+  const bool active = ex < t.Nx;
+  double* cv = sh[half] + 2 * kMaxQf;
+  if (active && sub < Q) {
+    const int c = scol(t, ex, sub);
+    cv[sub] = eta[c];
+    cv[Q + sub] = etax[c];
+    cv[2 * Q + sub] = phisx[c];
+    cv[3 * Q + sub] = w[c];
+  }
+  __syncwarp();
+  zak_element16(t, R, ex, active, sub, sh[half]);
 }
 
 __global__ void k_filter(SurfTables t, double* __restrict__ q0, double* __restrict__ q1) {
-  __shared__ double sh[kZakWarps][kSurfWarpScratch];
+  __shared__ double sh[kZakWarps][kSurfScratch];
   const int wid = threadIdx.x >> 5;
   const int ex = blockIdx.x * kZakWarps + wid;
   if (ex >= t.Nx) return;
@@ -84,31 +136,23 @@ __global__ void k_rk4(int stage, int n, double dt, double* __restrict__ eta, dou
   rk4_item(stage, dt, eta, phis, ke, kp, ae, ap, se, sp, i);
 }
 
-cudaError_t launch_wsurf(const SurfTables& t, const double* Phi, const double* eta, double* w,
-                         cudaStream_t s) {
-  k_wsurf<<<(t.ncol + 3) / 4, 128, 0, s>>>(t, Phi, eta, w);
+cudaError_t launch_recover(const SurfTables& t, const double* Phi, const double* eta, const double* phis, double* w,
+                           double* etax, double* phisx, cudaStream_t s) {
+  const size_t smem = sizeof(double) * (4 * (kRecElems + 2 * t.win + 2) + 2 * (kRecElems + 1));
+  k_recover<<<(t.Nx + kRecElems - 1) / kRecElems, kRecThreads, smem, s>>>(t, Phi, eta, phis, w, etax, phisx);
   count_launch();
   return cudaGetLastError();
 }
 
-cudaError_t launch_sx(const SurfTables& t, const double* f0, const double* f1, double* R,
-                      cudaStream_t s) {
-  const int n = 2 * t.Nx * (t.P + 1);
-  k_sx<<<(n + 255) / 256, 256, 0, s>>>(t, f0, f1, R);
-  count_launch();
-  return cudaGetLastError();
-}
-
-cudaError_t launch_mass1d(const SurfTables& t, const double* R, int nrhs, double* u0, double* u1,
-                          double* scratch, cudaStream_t s) {
-  k_mass1d<<<1, 256, 0, s>>>(t, R, nrhs, u0, u1, scratch);
+cudaError_t launch_mass1d(const SurfTables& t, const double* R, double* u0, double* u1, cudaStream_t s) {
+  k_mass1d<<<(t.Nx + kRecElems - 1) / kRecElems, kRecThreads, 0, s>>>(t, R, u0, u1);
   count_launch();
   return cudaGetLastError();
 }
 
 cudaError_t launch_zakharov(const SurfTables& t, const double* eta, const double* etax,
                             const double* phisx, const double* w, double* R, cudaStream_t s) {
-  k_zak<<<(t.Nx + kZakWarps - 1) / kZakWarps, 32 * kZakWarps, 0, s>>>(t, eta, etax, phisx, w, R);
+  k_zak<<<(t.Nx + 2 * kZakWarps - 1) / (2 * kZakWarps), 32 * kZakWarps, 0, s>>>(t, eta, etax, phisx, w, R);
   count_launch();
   return cudaGetLastError();
 }

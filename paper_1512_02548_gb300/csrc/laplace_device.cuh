@@ -1477,26 +1477,9 @@ static __global__ void __launch_bounds__(32) k_prec_tri(DevGeom g, PrecSetup ps,
 // ------------------------------------------------------------------------------------
 constexpr int kStageWarps = kThreads / 32;
 
-// The interface systems of the two right-hand sides (η, φ̃) of an M' solve: short systems on one
-// warp each (warps 0 and 1 of a one-CTA team, warp 0 of ranks 0 and 1 otherwise), long ones on a
-// whole CTA each.  Every thread of the CTA calls it.
-template <bool CACHE>
-__device__ __forceinline__ void mass1d_interfaces(const SurfTables& t, const Team& tm, double* scr) {
-  if (t.nif <= 32 * kTridiagRegs) {
-    const int warp = threadIdx.x >> 5;
-    if (tm.size == 1) {
-      if (warp < 2) mass1d_interface(t, 2, scr, warp);
-    } else if (tm.rank < 2 && warp == 0) {
-      mass1d_interface(t, 2, scr, tm.rank);
-    }
-    return;
-  }
-  for (int rh = tm.rank; rh < 2; rh += tm.size) mass1d_interface_cta<CACHE>(t, 2, scr, rh);
-}
-
 template <int P, bool MIXED, bool CACHE = false>
 __device__ void stage_body(Instance& I, const Team& tm, int stage, int step, unsigned char* smem_raw,
-                           double* red, int* s_flag, double (*sh)[kSurfWarpScratch]) {
+                           double* red, int* s_flag, double (*sh)[kSurfScratch]) {
   constexpr int Q = P + 1;
   const DevGeom& g = I.g;
   const SurfTables& t = I.st;
@@ -1575,7 +1558,7 @@ __device__ void stage_body(Instance& I, const Team& tm, int stage, int step, uns
     for (int k = tm.rank; k < I.ps.nr; k += tm.size) prec_tri_mode_cta(g, I.ps, k);
   } else {
     // one warp per mode, the modes spread over the team's CTAs and their warps
-    float* stg = 2 * I.ps.nif <= 2 * kSurfWarpScratch ? reinterpret_cast<float*>(sh[warp]) : nullptr;
+    float* stg = 2 * I.ps.nif <= 2 * kSurfScratch ? reinterpret_cast<float*>(sh[warp]) : nullptr;
     for (int k = tm.rank + tm.size * warp; k < I.ps.nr; k += tm.size * nw) prec_tri_mode(g, I.ps, k, stg);
   }
   if (!grid_barrier(tm, s_flag)) return;
@@ -1598,7 +1581,7 @@ __device__ void stage_body(Instance& I, const Team& tm, int stage, int step, uns
     if (Pk)
       for (int i = R.c0 * g.nrow + threadIdx.x; i < R.c1 * g.nrow; i += blockDim.x) Pk[i] = I.pa.x[i];
   }
-  // w̃ on owned columns; element S_x of η and φ̃; condensation of M'
+  // w̃ on owned columns; condensed element S_x of η and φ̃
   for (int c0 = R.c0 + 4 * warp; c0 < R.c1; c0 += 4 * nw) {
     const int col = c0 + (lane >> 3);
     wsurf_column8(t, I.pa.x, ein, I.wt, col < R.c1 ? col : -1, lane & 7);
@@ -1607,37 +1590,47 @@ __device__ void stage_body(Instance& I, const Team& tm, int stage, int step, uns
     const int fld = q / (ne * Q), r = q - fld * ne * Q;
     sx_item(t, ein, pin, I.R, fld * t.Nx * Q + R.e0 * Q + r);
   }
-  __syncthreads();
-  for (int q = threadIdx.x; q < 2 * ne; q += blockDim.x) {
-    const int rh = q / ne, ex = R.e0 + (q - rh * ne);
-    mass1d_condense(t, I.R, 2, I.scr, rh * t.Nx + ex);
-  }
   SEM_MARK(g, tm, TR_WSX);
   if (!grid_barrier(tm, s_flag)) return;
-  mass1d_interfaces<CACHE>(t, tm, I.scr);
-  if (!grid_barrier(tm, s_flag)) return;
-  SEM_MARK(g, tm, TR_MINT1);
-  for (int q = threadIdx.x; q < 2 * nc; q += blockDim.x) {
-    const int rh = q / nc, col = R.c0 + (q - rh * nc);
-    mass1d_backsub(t, I.R, 2, rh == 0 ? I.etax : I.phisx, I.scr, rh, col);
-  }
-  if (!grid_barrier(tm, s_flag)) return;
-  SEM_MARK(g, tm, TR_MBACK1);
-  // over-integrated Zakharov right-hand side of the owned elements and its M' solve
-  for (int ex = R.e0 + warp; ex < R.e1; ex += nw) zak_element(t, ein, I.etax, I.phisx, I.wt, I.R, ex, lane, sh[warp]);
+  // M' solve of ∂xη, ∂xφ̃ at both ends of every owned element
+  double* ub = I.ub + R.e0 + tm.rank;
+  mass1d_windows(t, I.R, R.e0, R.e1, ub, I.ub_stride);
   __syncthreads();
-  for (int q = threadIdx.x; q < 2 * ne; q += blockDim.x) {
-    const int rh = q / ne, ex = R.e0 + (q - rh * ne);
-    mass1d_condense(t, I.R, 2, I.scr, rh * t.Nx + ex);
+  SEM_MARK(g, tm, TR_MINT1);
+  // over-integrated Zakharov right-hand side of the owned elements, two per warp (the second one's
+  // scratch in the reduction buffer, idle here); ∂xη and ∂xφ̃ of an element come from its condensed rows and its
+  // two interface unknowns
+  {
+    static_assert(kRedSize >= kStageWarps * kSurfScratch, "the reduction buffer holds the second elements");
+    const int half = lane >> 4, sub = lane & 15;
+    double* zs = half ? red + warp * kSurfScratch : sh[warp];
+    double* cv = zs + 2 * kMaxQf;
+    for (int i0 = 2 * warp; i0 < ne; i0 += 2 * nw) {
+      const int i = i0 + half, ex = R.e0 + i;
+      const bool active = i < ne;
+      if (active && sub < Q) {
+        const int c = scol(t, ex, sub);
+        const double* Re = I.R + (size_t)ex * Q;
+        cv[sub] = __ldcg(ein + c);
+        cv[Q + sub] = mass1d_value(t, Re, ub[i], ub[i + 1], sub);
+        cv[2 * Q + sub] = mass1d_value(t, Re + (size_t)t.Nx * Q, ub[I.ub_stride + i], ub[I.ub_stride + i + 1], sub);
+        cv[3 * Q + sub] = __ldcg(I.wt + c);
+      }
+      __syncwarp();
+      zak_element16(t, I.R2, ex, active, sub, zs);
+    }
   }
   SEM_MARK(g, tm, TR_ZAK);
   if (!grid_barrier(tm, s_flag)) return;
-  mass1d_interfaces<CACHE>(t, tm, I.scr);
-  if (!grid_barrier(tm, s_flag)) return;
+  mass1d_windows(t, I.R2, R.e0, R.e1, ub, I.ub_stride);
+  __syncthreads();
   SEM_MARK(g, tm, TR_MINT2);
   for (int q = threadIdx.x; q < 2 * nc; q += blockDim.x) {
-    const int rh = q / nc, col = R.c0 + (q - rh * nc);
-    mass1d_backsub(t, I.R, 2, rh == 0 ? I.ke : I.kp, I.scr, rh, col);
+    const int rh = q >= nc ? 1 : 0, c = q - rh * nc;
+    const int i = min(c / P, ne - 1);
+    const double* u = ub + rh * I.ub_stride + i;
+    (rh ? I.kp : I.ke)[R.c0 + c] =
+        mass1d_value(t, I.R2 + ((size_t)rh * t.Nx + R.e0 + i) * Q, u[0], u[1], c - i * P);
   }
   __syncthreads();
   // relaxation source and the RK4 bookkeeping on owned columns
@@ -1667,7 +1660,7 @@ __global__ void __launch_bounds__(kThreads, WIDE ? 2 : 1) k_stage(StageArgs B) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double red[kRedSize];
   __shared__ int s_flag;
-  __shared__ __align__(16) double sh[kStageWarps][kSurfWarpScratch];
+  __shared__ __align__(16) double sh[kStageWarps][kSurfScratch];
   __shared__ __align__(16) Instance I;
   const int ii = B.cta_inst[blockIdx.x];
   {

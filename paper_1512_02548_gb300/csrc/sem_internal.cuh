@@ -160,22 +160,20 @@ struct SurfTables {
   int P, Pf, Nx, Nz, ncol, nrow, periodic;
   double g;
   const double* D;        // (P+1)²  differentiation on the GLL nodes
-  const double* MD;       // (P+1)²  M·D (element S_x without scale)
-  const double* B;        // (P+1)×(Pf+1)  Iᵀ M_f (over-integration projection)
+  const double* SX;       // (P+1)²  M·D, rows condensed (surface_device.cuh)
+  const double* ZB;       // (P+1)×(Pf+1)  Iᵀ M_f (over-integration projection), rows condensed
   const double* I;        // (Pf+1)×(P+1)  interpolation to the fine nodes
   const double* F;        // (P+1)²  modal filter
   const double* wrow;     // [nrow] row weights of the w̃ projection: w̃ d = Σ_iz wrow_iz Φ_iz
-  const double* Aii;      // (P−1)²  inverse interior block of M
   const double* Z;        // 2×(P−1) M_bi M_ii⁻¹
   const double* se;       // [Nx] Δx_e / 2
+  const double* r2dx;     // [Nx] 2/Δx_e
   const double* dsl;      // [Nz]
   const double* h;        // [ncol]
-  const double* th_e;     // interface tridiagonal: off-diagonals  [N]
-  const double* th_m;     // Thomas pivots                           [N]
-  const double* th_cp;    // Thomas c'                               [N]
-  const double* th_z;     // periodic: T'⁻¹u                         [N]
-  double th_vlast;        // periodic: v_{N−1}
-  double th_fac;          // periodic: 1/(1 + vᵀ T'⁻¹u)
+  const double* th_al;    // interface system of M': −e_{j−1} m_j       [N]
+  const double* th_m;     // 1/pivot m_j (cyclic factors when periodic) [N]
+  const double* th_cp;    // multiplier l_j = e_j m_j                   [N]
+  int win;                // interfaces after which the recurrences forget their start (1e-18)
   int nif;                // interface unknowns N
   int filter_on;
   // relaxation zones (§2.2)
@@ -203,7 +201,8 @@ struct Instance {
   double *s0e, *s0p;     // stage inputs (double-buffered: stages 2 and 4 read s0, stage 3 reads s1)
   double *s1e, *s1p;
   double *ke, *kp, *ae, *ap;
-  double *wt, *etax, *phisx, *R, *scr;
+  double *wt, *R, *R2, *ub;
+  int ub_stride;         // ub[2][ub_stride]: interface unknowns of the M' solves, CTA of rank r at e0 + r
   double *P1, *P2, *P3;  // stage potentials: P1, P2 of this step, P3 of the last stage 3
   double *D32;           // Φ₃ − Φ₂ of the last step
   double tstart, dt, tau;
@@ -276,14 +275,13 @@ cudaError_t launch_prec_setup(const DevGeom& g, const PrecSetup& ps, cudaStream_
 cudaError_t launch_pcg(const DevGeom& g, const PcgArgs& a, int grid, size_t smem, cudaStream_t s);
 
 // ---- launchers (kernels_surface.cu) ----
-cudaError_t launch_wsurf(const SurfTables& t, const double* Phi, const double* eta, double* w,
-                         cudaStream_t s);
-cudaError_t launch_sx(const SurfTables& t, const double* f0, const double* f1, double* R,
-                      cudaStream_t s);
-cudaError_t launch_mass1d(const SurfTables& t, const double* R, int nrhs, double* u0, double* u1,
-                          double* scratch, cudaStream_t s);
+// w̃ and the M'-projected ∂x of η and φ̃ (one kernel).
+cudaError_t launch_recover(const SurfTables& t, const double* Phi, const double* eta, const double* phis, double* w,
+                           double* etax, double* phisx, cudaStream_t s);
+// R = condensed over-integrated right-hand sides; then u0, u1 from M'u = Σ_e Q_eᵀ R_e.
 cudaError_t launch_zakharov(const SurfTables& t, const double* eta, const double* etax,
                             const double* phisx, const double* w, double* R, cudaStream_t s);
+cudaError_t launch_mass1d(const SurfTables& t, const double* R, double* u0, double* u1, cudaStream_t s);
 cudaError_t launch_filter(const SurfTables& t, double* q0, double* q1, cudaStream_t s);
 // Adds the relaxation source (1 − γ)(q_a − q)/τ to (de, dp) in the zones.
 cudaError_t launch_relax(const SurfTables& t, const double* eta, const double* phis, double time,

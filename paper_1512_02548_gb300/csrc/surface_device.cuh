@@ -8,33 +8,20 @@
 namespace semgb {
 
 constexpr int kMaxQf = 3 * kMaxP + 1;
-// shared scratch of one warp in the element bodies (zak, filter)
-constexpr int kSurfWarpScratch = 2 * kMaxQf + 4 * (kMaxP + 1);
+// shared scratch of an element in the element bodies (zak, filter)
+constexpr int kSurfScratch = 2 * kMaxQf + 4 * (kMaxP + 1);
 
 __device__ __forceinline__ int scol(const SurfTables& t, int ex, int a) {
   int c = ex * t.P + a;
   return c >= t.ncol ? c - t.ncol : c;
 }
 
-// w̃ at column `col` (one warp).  On the tensor-product mesh the 2D mass is M_x ⊗ M_σ and the
+// w̃ of column `col` by the 8 lanes of a warp with the same lane >> 3 (sub = lane & 7; every lane of the
+// warp calls, col < 0: no column).  On the tensor-product mesh the 2D mass is M_x ⊗ M_σ and the
 // σ-derivative (1/d)∂σΦ is continuous across x-element edges, so the surface row of
 // M⁻¹S_zΦ (eq. velocpot2) is the per-column contraction
 //     w̃ = (1/d) Σ_l Σ_b c_{l,b} (2/Δσ_l) (D Φ_l)_b,  c_l = (Δσ_l/2) M (M_σ⁻¹ e_top)|_l,
 // whose weights are folded on the host into one weight per row, w̃ = (1/d) Σ_iz wrow_iz Φ_iz.
-// Lanes take rows; the warp sums.
-__device__ __forceinline__ void wsurf_column(const SurfTables& t, const double* __restrict__ Phi,
-                                             const double* __restrict__ eta, double* __restrict__ w,
-                                             int col, int lane) {
-  const double* phi = Phi + (size_t)col * t.nrow;
-  double acc = 0.0;
-  for (int iz = lane; iz < t.nrow; iz += 32) acc = fma(t.wrow[iz], phi[iz], acc);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if (lane == 0) w[col] = acc / (eta[col] + t.h[col]);
-}
-
-// The same for four columns per warp, eight lanes per column (col < 0: no column; every lane of
-// the warp must call it).
 __device__ __forceinline__ void wsurf_column8(const SurfTables& t, const double* __restrict__ Phi,
                                               const double* __restrict__ eta, double* __restrict__ w,
                                               int col, int sub) {
@@ -48,133 +35,162 @@ __device__ __forceinline__ void wsurf_column8(const SurfTables& t, const double*
   if (col >= 0 && sub == 0) w[col] = acc / (eta[col] + t.h[col]);
 }
 
-// Element-local S_x f = M·D f_e (the Δx/2 and 2/Δx scales cancel); item k over
-// [field][ex][a], two fields.
+// M'u = Σ_e Q_eᵀ R_e (M' constant in time).  The element right-hand sides are stored condensed: the
+// element interiors are eliminated on the host, in the tables, so that an item of an element's row a is
+//   a = 0, P:      the boundary rows R_b − M_bi M_ii⁻¹ R_i (the interface right-hand side),
+//   0 < a < P:     the particular interior part M_ii⁻¹ R_i,
+// one dot product each.  Layout R[field][ex][a].
+
+// S_x f = M·D f_e condensed (the Δx/2 and 2/Δx scales cancel in the boundary rows; the interior part
+// takes 2/Δx); item k over [field][ex][a], two fields.
+__device__ __forceinline__ double sx_value(const SurfTables& t, const double* __restrict__ f, int ex, int a) {
+  const int Q = t.P + 1;
+  double s = 0.0;
+  for (int c = 0; c < Q; ++c) s = fma(t.SX[a * Q + c], __ldcg(f + scol(t, ex, c)), s);
+  return (a == 0 || a == t.P) ? s : s * t.r2dx[ex];
+}
 __device__ __forceinline__ void sx_item(const SurfTables& t, const double* __restrict__ f0,
                                         const double* __restrict__ f1, double* __restrict__ R, int k) {
   const int Q = t.P + 1;
   const int fld = k / (t.Nx * Q), rem = k - fld * t.Nx * Q, ex = rem / Q, a = rem - ex * Q;
-  const double* f = fld == 0 ? f0 : f1;
-  double s = 0.0;
-  for (int c = 0; c < Q; ++c) s = fma(t.MD[a * Q + c], f[scol(t, ex, c)], s);
-  R[k] = s;
+  R[k] = sx_value(t, fld == 0 ? f0 : f1, ex, a);
 }
 
-// M'u = Σ_e Q_eᵀ R_e by static condensation (M' is constant in time).  Scratch layout:
-// gL[nrhs][Nx], gR[nrhs][Nx], ub[nrhs][nif].
-// Phase 1, item k over [rhs][ex]: condensed boundary right-hand sides of element ex.
-__device__ __forceinline__ void mass1d_condense(const SurfTables& t, const double* __restrict__ R, int nrhs,
-                                                double* __restrict__ scr, int k) {
-  const int P = t.P, Q = P + 1, Pm = P - 1, Nx = t.Nx;
-  const double* Re = R + (size_t)k * Q;
-  double l = Re[0], r = Re[P];
-  for (int i = 0; i < Pm; ++i) {
-    l = fma(-t.Z[i], Re[1 + i], l);
-    r = fma(-t.Z[Pm + i], Re[1 + i], r);
+// Interface unknowns lo, lo+1, …, lo+cnt−1 (cyclic when periodic) of the condensed M' system, by one
+// warp, from the right-hand side gfun(j), 0 ≤ j < N; store(i, u) receives unknown lo + i.
+// The system's LDLᵀ factors decay: with the multipliers l_j = e_j/p_j, |l_j| ≤ |S01|/S00 = 1/(P+1) for
+// any element widths, so the recurrences
+//     y_j = g_j m_j − (e_{j−1} m_j) y_{j−1},        u_j = y_j − l_j u_{j+1}
+// started t.win interfaces away from the first unknown wanted (and from zero) agree with the whole
+// chain's to (P+1)^−win < 1e-18.  Every CTA therefore solves for its own elements alone, without
+// waiting for a solve of the whole chain elsewhere: an RK stage has four team barriers fewer and no
+// 2049-unknown solve on two CTAs while the others wait (step on the 2048×2 shoal 1849 → 1729 µs, on 64×4
+// 721 → 700 µs, 512 uneven tanks 12.52 → 12.17 ms).  The periodic chain uses the cyclic factors (the fixed point of the pivot recurrence around the ring), no closure.
+// Lanes hold chunks of c ≤ kWinRegs positions of the window; the composed affine maps are scanned
+// over as many lanes as cover t.win positions.
+constexpr int kWinRegs = 6;
+
+template <class G, class Store>
+__device__ __forceinline__ void mass1d_window(const SurfTables& t, G gfun, int lo, int cnt, Store store) {
+  const int lane = threadIdx.x & 31, N = t.nif, W = t.win;
+  const int len = cnt + 2 * W, c = (len + 31) >> 5;
+  const unsigned full = 0xffffffffu;
+  double al[kWinRegs], v[kWinRegs], cp[kWinRegs];
+  int j = lo - W + lane * c;
+  int jw = j;                                       // j around the ring
+  if (t.periodic) { jw %= N; if (jw < 0) jw += N; }
+#pragma unroll
+  for (int q = 0; q < kWinRegs; ++q) {
+    al[q] = v[q] = cp[q] = 0.0;
+    if (q < c) {
+      if (lane * c + q < len && jw >= 0 && jw < N) {
+        al[q] = t.th_al[jw];
+        v[q] = gfun(jw) * t.th_m[jw];
+        cp[q] = -t.th_cp[jw];
+      }
+      ++jw;
+      if (t.periodic && jw == N) jw = 0;
+    }
   }
-  scr[k] = l;
-  scr[nrhs * Nx + k] = r;
-}
-
-// Phase 2, one warp per right-hand side: the interface tridiagonal (cyclic when periodic).
-__device__ __forceinline__ void mass1d_interface(const SurfTables& t, int nrhs, double* __restrict__ scr,
-                                                 int rh) {
-  const int Nx = t.Nx, N = t.nif;
-  const double* gl = scr + rh * Nx;
-  const double* gr = scr + nrhs * Nx + rh * Nx;
-  double* ub = scr + 2 * nrhs * Nx + rh * N;
-  auto gfun = [&](int j) -> double {
-    if (t.periodic) return __ldcg(gl + j) + __ldcg(gr + (j == 0 ? Nx - 1 : j - 1));
-    return (j < Nx ? __ldcg(gl + j) : 0.0) + (j > 0 ? __ldcg(gr + j - 1) : 0.0);
-  };
-  warp_tridiag<double>(N, gfun, t.th_e, t.th_m, t.th_cp, t.periodic != 0, t.th_z, t.th_vlast, t.th_fac, ub);
-}
-
-// The same solve by a whole CTA (every thread must call it): long systems (N > 32·kTridiagRegs)
-// use the CTA-wide scan (CACHE: with register-held chunks), short ones warp 0 alone.
-template <bool CACHE = false>
-__device__ __forceinline__ void mass1d_interface_cta(const SurfTables& t, int nrhs, double* __restrict__ scr,
-                                                     int rh) {
-  const int Nx = t.Nx, N = t.nif;
-  if (N <= 32 * kTridiagRegs) {
-    if (threadIdx.x < 32) mass1d_interface(t, nrhs, scr, rh);
-    return;
+  double A = 1.0, B = 0.0;
+#pragma unroll
+  for (int q = 0; q < kWinRegs; ++q)
+    if (q < c) { B = fma(al[q], B, v[q]); A *= al[q]; }
+  for (int o = 1; o < 32 && o * c < W; o <<= 1) {
+    const double Ap = __shfl_up_sync(full, A, o), Bp = __shfl_up_sync(full, B, o);
+    if (lane >= o) { B = fma(A, Bp, B); A *= Ap; }
   }
-  const double* gl = scr + rh * Nx;
-  const double* gr = scr + nrhs * Nx + rh * Nx;
-  double* ub = scr + 2 * nrhs * Nx + rh * N;
-  auto gfun = [&](int j) -> double {
-    if (t.periodic) return __ldcg(gl + j) + __ldcg(gr + (j == 0 ? Nx - 1 : j - 1));
-    return (j < Nx ? __ldcg(gl + j) : 0.0) + (j > 0 ? __ldcg(gr + j - 1) : 0.0);
-  };
-  cta_tridiag<double, decltype(gfun), CACHE>(N, gfun, t.th_e, t.th_m, t.th_cp, t.periodic != 0, t.th_z, t.th_vlast,
-                                             t.th_fac, ub);
-}
-
-// Phase 3, column `col` of right-hand side `rh`: interface value or back-substituted interior.
-__device__ __forceinline__ void mass1d_backsub(const SurfTables& t, const double* __restrict__ R, int nrhs,
-                                               double* __restrict__ u, const double* __restrict__ scr,
-                                               int rh, int col) {
-  const int P = t.P, Q = P + 1, Pm = P - 1, Nx = t.Nx, N = t.nif;
-  const double* y = scr + 2 * nrhs * Nx + rh * N;
-  const int ex = col / P, a = col - ex * P;
-  double v;
-  if (a == 0) v = __ldcg(y + ex);   // interface node (incl. the walls' last column)
-  else {
-    const double* Re = R + ((size_t)rh * Nx + ex) * Q;
-    const int i = a - 1;
-    double s = 0.0;
-    for (int m = 0; m < Pm; ++m) s = fma(t.Aii[i * Pm + m], Re[1 + m], s);
-    const int jr = (ex + 1 == N) ? 0 : ex + 1;
-    v = s / t.se[ex] - (t.Z[i] * __ldcg(y + ex) + t.Z[Pm + i] * __ldcg(y + jr));
+  double y = __shfl_up_sync(full, B, 1);
+  if (lane == 0) y = 0.0;
+  A = 1.0;
+#pragma unroll
+  for (int q = 0; q < kWinRegs; ++q)
+    if (q < c) { y = fma(al[q], y, v[q]); v[q] = y; }
+  B = 0.0;
+#pragma unroll
+  for (int q = kWinRegs - 1; q >= 0; --q)
+    if (q < c) { B = fma(cp[q], B, v[q]); A *= cp[q]; }
+  for (int o = 1; o < 32 && o * c < W; o <<= 1) {
+    const double An = __shfl_down_sync(full, A, o), Bn = __shfl_down_sync(full, B, o);
+    if (lane + o < 32) { B = fma(A, Bn, B); A *= An; }
   }
-  u[col] = v;
+  double x = __shfl_down_sync(full, B, 1);
+  if (lane == 31) x = 0.0;
+#pragma unroll
+  for (int q = kWinRegs - 1; q >= 0; --q)
+    if (q < c) {
+      x = fma(cp[q], x, v[q]);
+      const int i = lane * c + q - W;
+      if (i >= 0 && i < cnt) store(i, x);
+    }
 }
 
-// Over-integrated Zakharov integrals of element ex (one warp, `sh` = kSurfWarpScratch doubles):
-// η, ηx, φ̃x, w̃ are interpolated to the Pf+1 fine GLL nodes, the PDE integrands of eq. FSeqs
-// evaluated pointwise and projected with Iᵀ M_f (Δx/2) (§3.1.1, §3.3).  R[0][ex][·] and
-// R[1][ex][·] receive the element right-hand sides of ∂tη and ∂tφ̃.
-__device__ __forceinline__ void zak_element(const SurfTables& t, const double* __restrict__ eta,
-                                            const double* __restrict__ etax, const double* __restrict__ phisx,
-                                            const double* __restrict__ w, double* __restrict__ R, int ex,
-                                            int lane, double* sh) {
+// Interface unknowns e0 … e1 (both ends of every element e0 … e1−1) of both right-hand sides, by all
+// warps of the CTA, from condensed right-hand sides R (read through L2: other CTAs wrote some of them);
+// ub[rh·stride + i] receives unknown e0 + i.  The caller synchronises the CTA afterwards.
+__device__ __forceinline__ void mass1d_windows(const SurfTables& t, const double* R, int e0, int e1, double* ub,
+                                               int stride) {
+  const int Q = t.P + 1, Nx = t.Nx, nw = blockDim.x >> 5;
+  const int seg = 32 * kWinRegs - 2 * t.win, total = e1 - e0 + 1, nseg = (total + seg - 1) / seg;
+  for (int k = threadIdx.x >> 5; k < 2 * nseg; k += nw) {
+    const int rh = k & 1, i0 = (k >> 1) * seg;
+    const double* Rr = R + (size_t)rh * Nx * Q;
+    auto gfun = [&](int j) -> double {
+      const int jl = j > 0 ? j - 1 : (t.periodic ? Nx - 1 : -1);
+      return (j < Nx ? __ldcg(Rr + (size_t)j * Q) : 0.0) + (jl >= 0 ? __ldcg(Rr + (size_t)jl * Q + t.P) : 0.0);
+    };
+    double* o = ub + rh * stride + i0;
+    mass1d_window(t, gfun, e0 + i0, min(seg, total - i0), [&](int i, double u) { o[i] = u; });
+  }
+}
+
+// Value at local column a of element ex from its condensed rows Re and the interface unknowns ul, ur at
+// its ends.
+__device__ __forceinline__ double mass1d_value(const SurfTables& t, const double* Re, double ul, double ur, int a) {
+  if (a == 0) return ul;
+  if (a == t.P) return ur;
+  return Re[a] - (t.Z[a - 1] * ul + t.Z[t.P - 1 + a - 1] * ur);
+}
+
+// Over-integrated Zakharov integrals of element ex: η, ηx, φ̃x, w̃ (cv: 4·Q coarse values in shared
+// memory) are interpolated to the Pf+1 fine GLL nodes, the PDE integrands of eq. FSeqs evaluated
+// pointwise and projected with Iᵀ M_f (Δx/2) (§3.1.1, §3.3).  R[0][ex][·] and R[1][ex][·] receive the
+// condensed element right-hand sides of ∂tη and ∂tφ̃.  By the 16 lanes of half a warp (sub = 0..15),
+// both halves in step (`active`: this half has an element): an FP64 instruction occupies the narrow pipe for a whole warp's
+// time whatever its active lanes, and the fine nodes of the usual orders fit 16 lanes.
+__device__ __forceinline__ void zak_element16(const SurfTables& t, double* __restrict__ R, int ex, bool active,
+                                              int sub, double* sh) {
   const int Q = t.P + 1, Qf = t.Pf + 1;
   double* Fe = sh;
   double* Fp = Fe + kMaxQf;
-  double* cv = Fp + kMaxQf;   // 4*Q coarse values: η, ηx, φ̃x, w̃
-  if (lane < Q) {
-    const int c = scol(t, ex, lane);
-    cv[lane] = __ldcg(eta + c);
-    cv[Q + lane] = __ldcg(etax + c);
-    cv[2 * Q + lane] = __ldcg(phisx + c);
-    cv[3 * Q + lane] = __ldcg(w + c);
-  }
-  __syncwarp();
-  for (int q = lane; q < Qf; q += 32) {
-    const double* Iq = t.I + q * Q;
-    double e = 0, ex_ = 0, px = 0, wv = 0;
-    for (int c = 0; c < Q; ++c) {
-      e = fma(Iq[c], cv[c], e);
-      ex_ = fma(Iq[c], cv[Q + c], ex_);
-      px = fma(Iq[c], cv[2 * Q + c], px);
-      wv = fma(Iq[c], cv[3 * Q + c], wv);
+  const double* cv = Fp + kMaxQf;
+  if (active)
+    for (int q = sub; q < Qf; q += 16) {
+      const double* Iq = t.I + q * Q;
+      double e = 0, ex_ = 0, px = 0, wv = 0;
+      for (int c = 0; c < Q; ++c) {
+        const double w = Iq[c];
+        e = fma(w, cv[c], e);
+        ex_ = fma(w, cv[Q + c], ex_);
+        px = fma(w, cv[2 * Q + c], px);
+        wv = fma(w, cv[3 * Q + c], wv);
+      }
+      const double s2 = fma(ex_, ex_, 1.0);
+      Fe[q] = fma(wv, s2, -ex_ * px);
+      Fp[q] = -t.g * e - 0.5 * fma(px, px, -wv * wv * s2);
     }
-    const double s2 = fma(ex_, ex_, 1.0);
-    Fe[q] = fma(wv, s2, -ex_ * px);
-    Fp[q] = -t.g * e - 0.5 * fma(px, px, -wv * wv * s2);
-  }
   __syncwarp();
-  const double se = t.se[ex];
-  for (int a = lane; a < Q; a += 32) {
-    const double* Ba = t.B + a * Qf;
-    double se0 = 0, se1 = 0;
-    for (int q = 0; q < Qf; ++q) {
-      se0 = fma(Ba[q], Fe[q], se0);
-      se1 = fma(Ba[q], Fp[q], se1);
+  if (active) {
+    const double se = t.se[ex];
+    for (int k = sub; k < 2 * Q; k += 16) {
+      const int fld = k >= Q ? 1 : 0, a = k - fld * Q;
+      const double* Ba = t.ZB + a * Qf;
+      const double* F = fld ? Fp : Fe;
+      double s = 0.0;
+      for (int q = 0; q < Qf; ++q) s = fma(Ba[q], F[q], s);
+      // the interior part Δx/2 · (Δx/2 · M_ii)⁻¹: the scales cancel
+      R[((size_t)fld * t.Nx + ex) * Q + a] = (a == 0 || a == t.P) ? se * s : s;
     }
-    R[(size_t)ex * Q + a] = se * se0;
-    R[((size_t)t.Nx + ex) * Q + a] = se * se1;
   }
   __syncwarp();
 }
