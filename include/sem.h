@@ -170,7 +170,9 @@ int sem_laplace_apply(sem_mesh* m, const double* x_d, double* y_d, void* stream)
 /* The same operator in FP32 (the arithmetic of the mixed-precision inner solve): y = 𝓛 x
  * with the FP32 copy of the geometry of the last sem_update_geometry.  One kernel, tiles of
  * consecutive x-elements with the element left of each tile recomputed, so every output
- * column is complete in one CTA and written once; uses no workspace.  x_d, y_d: device,
+ * column is complete in one CTA and written once; uses no workspace.  Orders up to 8 with up to
+ * four layers take one element per thread (7 and 8 from a few thousand elements on), others
+ * line passes through shared memory.  x_d, y_d: device,
  * float, n values, must not overlap.  The environment variable SEM_APPLY_F32=tc selects, for
  * orders 4..7, a kernel whose element contractions run on the tensor cores (TF32 products
  * split three ways for FP32 accuracy; same result up to rounding, and slower on GB300). */
@@ -307,8 +309,8 @@ typedef struct sem_batch_tuning {
 } sem_batch_tuning;
 int sem_set_batch_tuning(const sem_batch_tuning* t);
 int sem_get_batch_tuning(sem_batch_tuning* t);
-/* Tile width (elements per tile, 1..16) of the FP32 tiled apply (sem_laplace_apply_f32, CUDA-core
- * kernel) for order P and Nz layers, as measured by the autotuner; 0 restores the default (the widest
+/* Tile width (elements per tile, 1..16) of the FP32 apply by line passes (sem_laplace_apply_f32 where it
+ * does not take one element per thread) for order P and Nz layers, as measured by the autotuner; 0 restores the default (the widest
  * tile up to 16 that keeps three CTAs per SM).  The FP64 apply takes the widest tile up to 16 that
  * fits in shared memory.  Process-wide. */
 int sem_set_apply_tile_width(int P, int Nz, int E);

@@ -344,7 +344,9 @@ __global__ void __launch_bounds__(kThreads) k_apply(DevGeom g, const double* __r
 
 }  // namespace semgb
 
+#include "even_odd.cuh"
 #include "apply_tile.cuh"
+#include "apply_elem.cuh"
 #include "apply_tc.cuh"
 
 namespace semgb {
@@ -1688,6 +1690,19 @@ cudaError_t upload_tables_impl(const double* D64, const double* w64) {
   if ((e = cudaMemcpyToSymbol(c_D64, D64, sizeof(double) * kDTotal)) != cudaSuccess) return e;
   if ((e = cudaMemcpyToSymbol(c_D32, D32, sizeof(float) * kDTotal)) != cudaSuccess) return e;
   if ((e = cudaMemcpyToSymbol(c_w64, w64, sizeof(double) * kWTotal)) != cudaSuccess) return e;
+  constexpr int Q = P + 1;
+  const double* D = D64 + d_off(P);
+  const double* w = w64 + w_off(P);
+  double H[Q * Q];
+  for (int i = 0; i < Q; ++i)
+    for (int j = 0; j < Q; ++j) H[i * Q + j] = D[j * Q + i] * w[j];
+  EoTables eo{};
+  fill_eo<P>(eo.D64, D, 1.0);
+  fill_eo<P>(eo.H64, H, 1.0);
+  fill_eo<P>(eo.D32, D, 1.0);
+  fill_eo<P>(eo.Dh32, D, 0.5);
+  fill_eo<P>(eo.H32, H, 1.0);
+  if ((e = cudaMemcpyToSymbol(c_eo, &eo, sizeof(eo))) != cudaSuccess) return e;
   return cudaMemcpyToSymbol(c_w32, w32, sizeof(float) * kWTotal);
 }
 
@@ -1819,12 +1834,12 @@ cudaError_t launch_stage_cluster_impl(int mixed, int wide, const StageArgs& a, i
 constexpr size_t kTileSmemTarget = 76 * 1024;
 
 template <int P>
-static int tile_grid(const void* fn, size_t smem, int E, int Nx, int slot, cudaError_t* err) {
+static int tile_grid(const void* fn, size_t smem, int E, int Nx, int slot, cudaError_t* err, int threads = kThreads) {
   // the attribute, the SM count and the occupancy for the last (device, smem) of each kernel
   // variant are kept, so that a repeated apply costs one launch on the host
   static std::mutex mu;
-  static int last_dev[9] = {-1, -1, -1, -1, -1, -1, -1, -1, -1}, last_sms[9] = {0}, last_per_sm[9] = {0};
-  static size_t last_smem[9] = {0};
+  static int last_dev[13] = {-1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1, -1}, last_sms[13] = {0}, last_per_sm[13] = {0};
+  static size_t last_smem[13] = {0};
   int dev = 0, sms = 0, per_sm = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) { *err = e; return 0; }
@@ -1833,7 +1848,7 @@ static int tile_grid(const void* fn, size_t smem, int E, int Nx, int slot, cudaE
     if (last_dev[slot] != dev || last_smem[slot] != smem) {
       if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem)) != cudaSuccess ||
           (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
-          (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kThreads, smem)) != cudaSuccess) {
+          (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem)) != cudaSuccess) {
         *err = e;
         return 0;
       }
@@ -1846,6 +1861,28 @@ static int tile_grid(const void* fn, size_t smem, int E, int Nx, int slot, cudaE
   const long long ntiles = (Nx + E - 1) / E;
   *err = cudaSuccess;
   return (int)(ntiles < (long long)per_sm * sms ? ntiles : (long long)per_sm * sms);
+}
+
+// The one-element-per-thread FP32 kernel (apply_elem.cuh): orders up to 8 (beyond, an element's values and
+// results no longer fit in a thread's registers), up to four layers.
+constexpr int kElemMaxP = 8;
+
+template <int P>
+static bool elem_fills(const DevGeom& g) {
+  const int E = g.Nz == 1 ? ElemTile<P, 1>::E : g.Nz == 2 ? ElemTile<P, 2>::E : g.Nz == 3 ? ElemTile<P, 3>::E : ElemTile<P, 4>::E;
+  return g.Nx >= 152 * E;
+}
+
+template <int P, int NZ>
+static cudaError_t launch_apply_elem(const DevGeom& g, const float* x, float* y, int bulk_ok, int vec_ok, cudaStream_t s) {
+  using L = ElemTile<P, NZ>;
+  cudaError_t e = cudaSuccess;
+  const void* fn = (const void*)k_apply_elem<P, NZ>;
+  const int grid = tile_grid<P>(fn, L::smem, L::E, g.Nx, 9 + NZ - 1, &e, L::threads);
+  if (e != cudaSuccess) return e;
+  k_apply_elem<P, NZ><<<grid, L::threads, L::smem, s>>>(g, x, y, bulk_ok, vec_ok);
+  count_launch();
+  return cudaGetLastError();
 }
 
 template <int P>
@@ -1874,6 +1911,19 @@ cudaError_t launch_apply_tile_impl(int fp32, const DevGeom& g, const void* x, vo
       }
       count_launch();
       return cudaGetLastError();
+    }
+  }
+  if constexpr (P <= kElemMaxP) {
+    // one element per thread; orders 7 and 8 (255 registers, 2 CTAs an SM) from the size on that gives
+    // every SM a tile: 2.5 M nodes at P = 8 take 23–27 → 17–23 µs, 0.6 M nodes 10–12 → 14–16
+    if (fp32 && g.Nz <= 4 && (P <= 6 || elem_fills<P>(g))) {
+      const int vec_ok = (reinterpret_cast<uintptr_t>(y) % 16) == 0 ? 1 : 0;
+      switch (g.Nz) {
+        case 1: return launch_apply_elem<P, 1>(g, xf, yf, bulk_ok, vec_ok, s);
+        case 2: return launch_apply_elem<P, 2>(g, xf, yf, bulk_ok, vec_ok, s);
+        case 3: return launch_apply_elem<P, 3>(g, xf, yf, bulk_ok, vec_ok, s);
+        default: return launch_apply_elem<P, 4>(g, xf, yf, bulk_ok, vec_ok, s);
+      }
     }
   }
   const size_t elem = fp32 ? sizeof(float) : sizeof(double);
