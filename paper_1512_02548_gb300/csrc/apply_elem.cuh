@@ -177,11 +177,11 @@ __global__ void __launch_bounds__(ElemTile<P, NZ>::threads, ElemTile<P, NZ>::cta
         float r1[Q], r2[Q], t1[Q], t2[Q], F1a[Q], F2a[Q], F1b[Q], F2b[Q];
 #pragma unroll
         for (int b = 0; b < Q; ++b) {
-          float S = c_eo.D32.O[i * h] * u[P][b], V = c_eo.D32.E[i * h] * u[0][b];
+          float S = c_eo.D32.O[i * eo_stride(Q)] * u[P][b], V = c_eo.D32.E[i * eo_stride(Q)] * u[0][b];
 #pragma unroll
           for (int j = 1; j < h; ++j) {
-            S = fmaf(c_eo.D32.O[i * h + j], u[P - j][b], S);
-            V = fmaf(c_eo.D32.E[i * h + j], u[j][b], V);
+            S = fmaf(c_eo.D32.O[i * eo_stride(Q) + j], u[P - j][b], S);
+            V = fmaf(c_eo.D32.E[i * eo_stride(Q) + j], u[j][b], V);
           }
           if constexpr (Q % 2) V = fmaf(c_eo.D32.C[i], u[h][b], V);
           r1[b] = S + V;
@@ -198,8 +198,8 @@ __global__ void __launch_bounds__(ElemTile<P, NZ>::threads, ElemTile<P, NZ>::cta
           const float fe = F1a[b] + F1b[b], fo = F1a[b] - F1b[b];
 #pragma unroll
           for (int c = 0; c < h; ++c) {
-            yv[c][b] = fmaf(c_eo.H32.O[c * h + i], fo, yv[c][b]);          // S_c
-            yv[P - c][b] = fmaf(c_eo.H32.E[c * h + i], fe, yv[P - c][b]);  // T_c
+            yv[c][b] = fmaf(c_eo.H32.O[c * eo_stride(Q) + i], fo, yv[c][b]);          // S_c
+            yv[P - c][b] = fmaf(c_eo.H32.E[c * eo_stride(Q) + i], fe, yv[P - c][b]);  // T_c
           }
           if constexpr (Q % 2) yv[h][b] = fmaf(c_eo.H32.R[i], fo, yv[h][b]);
           const float p = F2a[b], q = F2b[b];

@@ -16,6 +16,9 @@
 // periodic end, or whose rounded range would pass the end of x, are staged with plain loads.
 //
 // Per tile, with the tile's nodal values staged in shared memory:
+// Every contraction is taken in its even-odd form (even_odd.cuh): FP64, which holds the narrow FP64 pipe,
+// needs about 42 operations per node instead of 54, and two CTAs per SM cover each other's barriers:
+// 30011×2, P = 7: 424 → 320 µs; 8 M nodes, P = 4..10: 20–40% less.
 //   1. x-lines (element e, layer l, row b): u_r(a) = Σ_c D_ac u(c,b) for all a, in registers;
 //   2. σ-lines (e, l, column a): u_t(b) = Σ_c D_bc u(a,c); the geometric factors of column a
 //      (d, 1/d, ∂xh, ∂xd) and the layer ratios give
@@ -144,13 +147,21 @@ static __device__ __forceinline__ bool tile_range(const DevGeom& g, int ex0, int
   return true;
 }
 
+// FP64: two CTAs per SM, so that one CTA's FP64 work covers the other's barriers and staging: of 256
+// threads at 128 registers up to order 6, of 192 threads at 168 registers for orders 7 and 8 (fewer
+// would spill); one CTA of 256 beyond.
+template <int P, class T>
+constexpr int tile_threads() { return sizeof(T) == 8 && (P == 7 || P == 8) ? 192 : kThreads; }
+template <int P, class T>
+constexpr int tile_ctas() { return sizeof(T) == 8 && P <= 8 ? 2 : 0; }
+
 // bulk_ok != 0: x is 16-byte aligned and interior tiles are staged by bulk copies.
 // NZC > 0: the layer count is the compile-time constant NZC (= g.Nz), which turns the row
 // arithmetic into constants; NZC = 0 reads it from g.
 // Minimum of 3 CTAs per SM (at most 85 registers) only for FP32, P = 8, four layers, which the
 // compiler otherwise builds with 96 registers (two CTAs per SM); 0 leaves the choice to it.
 template <int P, class T, int NZC>
-__global__ void __launch_bounds__(kThreads, (sizeof(T) == 4 && P == 8 && NZC == 4) ? 3 : 0)
+__global__ void __launch_bounds__(tile_threads<P, T>(), (sizeof(T) == 4 && P == 8 && NZC == 4) ? 3 : tile_ctas<P, T>())
     k_apply_tile(DevGeom g, const T* __restrict__ x, T* __restrict__ y,
                                                          int E, int bulk_ok) {
   constexpr int Q = P + 1;
@@ -171,8 +182,7 @@ __global__ void __launch_bounds__(kThreads, (sizeof(T) == 4 && P == 8 && NZC == 
   T* Rrow = Ws + Q;                         // [en][Nz][Q] top-row (b = P) contributions, a < P
   T* Ccol = Rrow + (size_t)L.en_max * Nz * Q;   // [en][Nz][Q] right-column (a = P) contributions
   __shared__ int s_ok;
-  const T* D = CT<T>::D() + d_off(P);       // compile-time indices only: constant operands
-  const T* w = CT<T>::w() + w_off(P);
+  const T* w = CT<T>::w() + w_off(P);       // compile-time indices only: constant operands
   const T* geo = geo_ptr<T>(g);
   for (int t = threadIdx.x; t < nrow; t += blockDim.x) Ss[t] = (T)g.sig[t];
   for (int t = threadIdx.x; t < Q; t += blockDim.x) Ws[t] = w[t];
@@ -240,8 +250,9 @@ __global__ void __launch_bounds__(kThreads, (sizeof(T) == 4 && P == 8 && NZC == 
         if (gc < 0) gc = g.periodic ? gc + ncol : -1;
         else if (gc >= ncol) gc -= ncol;         // periodic: column Nx·P is column 0
         const T* xc = x + (size_t)(gc < 0 ? 0 : gc) * nrow;
-        for (int r = lane; r < nrow; r += 32) X[j * nrow + r] = gc >= 0 ? __ldg(xc + r) : T(0);
+        for (int r = lane; r < nrow; r += 32) cp_async1(X + j * nrow + r, xc + r, gc >= 0);
       }
+      cp_async_wait();
     }
     for (int t = threadIdx.x; t < en * Q * 4; t += blockDim.x) {
       const int e = t / (Q * 4);
@@ -253,14 +264,15 @@ __global__ void __launch_bounds__(kThreads, (sizeof(T) == 4 && P == 8 && NZC == 
       const int e = t / Nz, l = t - e * Nz;
       int ge = ex0 - 1 + e;
       if (ge < 0) ge = g.periodic ? ge + Nx : 0;
-      const T dxe = (T)g.dxe[ge], dsl = (T)g.dsl[l];   // ratios in the kernel's own precision
-      Cs[2 * t] = dsl / dxe;
-      Cs[2 * t + 1] = dxe / dsl;
+      const double* cz = g.cxz + ((size_t)ge * Nz + l) * 2;
+      Cs[2 * t] = (T)cz[0];
+      Cs[2 * t + 1] = (T)cz[1];
     }
     __syncthreads();
     if (!s_ok) break;                            // a copy did not complete: stop (status set below)
     const int e_first = has_left ? 0 : 1;        // walls: no element left of x = 0
     // ---- 1. x-lines: u_r ----
+#pragma unroll 1
     for (int e = e_first + le0, rem = lr0; e < en; e += lde, rem += ldr) {
       if (rem >= lpe) { rem -= lpe; ++e; if (e >= en) break; }
       const int l = rem / Q, bb = rem - l * Q;
@@ -269,16 +281,14 @@ __global__ void __launch_bounds__(kThreads, (sizeof(T) == 4 && P == 8 && NZC == 
 #pragma unroll
       for (int c = 0; c < Q; ++c) u[c] = Xl[c * nrow];
       T* out = Ur + (e * Nz + l) * BS + bb * QP;
+      T r[Q];
+      eo_line<Q, T>(eo_D<T>(), u, r);
 #pragma unroll
-      for (int a = 0; a < Q; ++a) {
-        T s = T(0);
-#pragma unroll
-        for (int c = 0; c < Q; ++c) s = fmx(D[a * Q + c], u[c], s);
-        out[a] = s;
-      }
+      for (int a = 0; a < Q; ++a) out[a] = r[a];
     }
     __syncthreads();
     // ---- 2. σ-lines: u_t, F1, F2 and the σ part of the transpose ----
+#pragma unroll 1
     for (int e = e_first + le0, rem = lr0; e < en; e += lde, rem += ldr) {
       if (rem >= lpe) { rem -= lpe; ++e; if (e >= en) break; }
       const int l = rem / Q, a = rem - l * Q;
@@ -289,30 +299,22 @@ __global__ void __launch_bounds__(kThreads, (sizeof(T) == 4 && P == 8 && NZC == 
       const T* gq = Gs + (e * Q + a) * 4;
       const T c0 = Cs[2 * (e * Nz + l)], c1 = Cs[2 * (e * Nz + l) + 1];
       const T wa = Ws[a], hx = gq[2], dxd = gq[3];
-      const T g11 = wa * c0 * gq[0];             // w_a Δσ/Δx d
-      const T g22 = wa * c1 * gq[1];             // w_a Δx/Δσ /d
+      const T g11 = c0 * gq[0];                  // Δσ/Δx d
+      const T g22 = c1 * gq[1];                  // Δx/Δσ /d
       const T* sg = Ss + l * P;
       const int base = (e * Nz + l) * BS;
-      T f2[Q];
+      T ut[Q], f2[Q];
+      eo_line<Q, T>(eo_D<T>(), u, ut);
 #pragma unroll
-      for (int bb = 0; bb < Q; ++bb) {
-        T ut = T(0);
-#pragma unroll
-        for (int c = 0; c < Q; ++c) ut = fmx(D[bb * Q + c], u[c], ut);
+      for (int bb = 0; bb < Q; ++bb) {           // F1/w_a and F2/(w_a w_b): the weights are in the tables of H
         const T ur = Ur[base + bb * QP + a];
         const T K12 = fmx(-sg[bb], dxd, hx);
-        const T wb = w[bb];
-        const T G12 = wa * wb * K12;
-        Fs[base + bb * QP + a] = fmx(g11 * wb, ur, G12 * ut);
-        f2[bb] = fmx(G12, ur, g22 * wb * fmx(K12, K12, T(1)) * ut);
+        Fs[base + bb * QP + a] = w[bb] * fmx(g11, ur, K12 * ut[bb]);
+        f2[bb] = fmx(K12, ur, g22 * fmx(K12, K12, T(1)) * ut[bb]);
       }
+      eo_line<Q, T>(eo_H<T>(), f2, ut);
 #pragma unroll
-      for (int bb = 0; bb < Q; ++bb) {
-        T s = T(0);
-#pragma unroll
-        for (int c = 0; c < Q; ++c) s = fmx(D[c * Q + bb], f2[c], s);
-        Ys[base + bb * QP + a] = s;
-      }
+      for (int bb = 0; bb < Q; ++bb) Ys[base + bb * QP + a] = wa * ut[bb];
     }
     __syncthreads();
     // ---- 3. x-lines: element contributions into the tile's nodes ----
@@ -323,6 +325,7 @@ __global__ void __launch_bounds__(kThreads, (sizeof(T) == 4 && P == 8 && NZC == 
     // and the right column of an element (a = P) go to small buffers and are added afterwards,
     // rows first, then columns.
     T* Yt = Ur;
+#pragma unroll 1
     for (int e = e_first + le0, rem = lr0; e < en; e += lde, rem += ldr) {
       if (rem >= lpe) { rem -= lpe; ++e; if (e >= en) break; }
       const int l = rem / Q, bb = rem - l * Q;
@@ -332,11 +335,11 @@ __global__ void __launch_bounds__(kThreads, (sizeof(T) == 4 && P == 8 && NZC == 
       for (int c = 0; c < Q; ++c) f1[c] = Fs[row + c];
       const bool top = bb == P && l < Nz - 1;   // row shared with the layer above
       T* yn = Yt + (e * P) * nrow + l * P + bb;
+      T y1[Q];
+      eo_line<Q, T>(eo_H<T>(), f1, y1);
 #pragma unroll
       for (int a = 0; a < Q; ++a) {
-        T s = Ys[row + a];
-#pragma unroll
-        for (int c = 0; c < Q; ++c) s = fmx(D[c * Q + a], f1[c], s);
+        const T s = Ys[row + a] + y1[a];
         if (a == P) Ccol[(e * Nz + l) * Q + bb] = s;
         else if (top) Rrow[(e * Nz + l) * Q + a] = s;
         else yn[a * nrow] = s;

@@ -13,9 +13,12 @@ namespace semgb {
 
 // Tables of the translation unit's order: O, E (h×h), C, R (h) of a matrix with that symmetry.
 constexpr int kEoH = (kMaxP + 1) / 2;
+// Rows of odd length: rows of whole 16-byte multiples would be loaded into registers as vectors, two tables
+// of them through a loop (118 instead of 44 registers for two lines of 8), instead of being operands.
+__host__ __device__ constexpr int eo_stride(int Q) { return Q / 2 | 1; }
 template <class T>
 struct EoTable {
-  T O[kEoH * kEoH], E[kEoH * kEoH], C[kEoH], R[kEoH];
+  T O[kEoH * (kEoH | 1)], E[kEoH * (kEoH | 1)], C[kEoH], R[kEoH];
 };
 struct EoTables {
   EoTable<double> D64, H64;        // D and H = Dᵀ W
@@ -34,8 +37,8 @@ static void fill_eo(EoTable<T>& t, const double* M, double scale) {   // M: Q×Q
   constexpr int Q = P + 1, h = Q / 2;
   for (int i = 0; i < h; ++i) {
     for (int j = 0; j < h; ++j) {
-      t.O[i * h + j] = (T)(scale * 0.5 * (M[i * Q + j] - M[i * Q + P - j]));
-      t.E[i * h + j] = (T)(scale * 0.5 * (M[i * Q + j] + M[i * Q + P - j]));
+      t.O[i * eo_stride(Q) + j] = (T)(scale * 0.5 * (M[i * Q + j] - M[i * Q + P - j]));
+      t.E[i * eo_stride(Q) + j] = (T)(scale * 0.5 * (M[i * Q + j] + M[i * Q + P - j]));
     }
     t.C[i] = Q % 2 ? (T)(scale * M[i * Q + h]) : T(0);
     t.R[i] = Q % 2 ? (T)(scale * M[h * Q + i]) : T(0);
@@ -51,9 +54,9 @@ __device__ __forceinline__ void eo_line(const EoTable<T>& t, const T (&u)[Q], T 
   for (int j = 0; j < h; ++j) { e[j] = u[j] + u[P - j]; o[j] = u[j] - u[P - j]; }
 #pragma unroll
   for (int i = 0; i < h; ++i) {
-    T S = t.O[i * h] * o[0], V = t.E[i * h] * e[0];
+    T S = t.O[i * eo_stride(Q)] * o[0], V = t.E[i * eo_stride(Q)] * e[0];
 #pragma unroll
-    for (int j = 1; j < h; ++j) { S = fmx(t.O[i * h + j], o[j], S); V = fmx(t.E[i * h + j], e[j], V); }
+    for (int j = 1; j < h; ++j) { S = fmx(t.O[i * eo_stride(Q) + j], o[j], S); V = fmx(t.E[i * eo_stride(Q) + j], e[j], V); }
     if constexpr (Q % 2) V = fmx(t.C[i], u[h], V);
     out[i] = S + V;
     out[P - i] = S - V;

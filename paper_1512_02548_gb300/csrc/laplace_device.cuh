@@ -1927,8 +1927,8 @@ cudaError_t launch_apply_tile_impl(int fp32, const DevGeom& g, const void* x, vo
     }
   }
   const size_t elem = fp32 ? sizeof(float) : sizeof(double);
-  // the FP64 kernel holds one CTA per SM (its registers), so only the shared-memory maximum caps it
-  const size_t cap = fp32 ? kTileSmemTarget : (size_t)kMaxDynSmem;
+  // three (FP32) or two CTAs per SM (FP64, orders up to 8; beyond, only the shared-memory maximum caps the tile)
+  const size_t cap = fp32 ? kTileSmemTarget : tile_ctas<P, double>() == 2 ? (size_t)112 * 1024 : (size_t)kMaxDynSmem;
   int E = 16;
   while (E > 1 && apply_tile_smem<P>(E, g.nrow, g.Nz, elem) > cap) E >>= 1;
   const int Et = fp32 ? apply_tile_width(P, g.Nz) : 0;   // a measured FP32 width (autotuner), if set
@@ -1941,10 +1941,10 @@ cudaError_t launch_apply_tile_impl(int fp32, const DevGeom& g, const void* x, vo
   const void* fns[5] = {(const void*)k_apply_tile<P, double, 0>, (const void*)k_apply_tile<P, float, 0>,
                         (const void*)k_apply_tile<P, float, 1>, (const void*)k_apply_tile<P, float, 2>,
                         (const void*)k_apply_tile<P, float, 4>};
-  const int grid = tile_grid<P>(fns[k], smem, E, g.Nx, k, &e);
+  const int grid = tile_grid<P>(fns[k], smem, E, g.Nx, k, &e, fp32 ? kThreads : tile_threads<P, double>());
   if (e != cudaSuccess) return e;
   switch (k) {
-    case 0: k_apply_tile<P, double, 0><<<grid, kThreads, smem, s>>>(g, static_cast<const double*>(x),
+    case 0: k_apply_tile<P, double, 0><<<grid, tile_threads<P, double>(), smem, s>>>(g, static_cast<const double*>(x),
                                                                    static_cast<double*>(y), E, bulk_ok); break;
     case 1: k_apply_tile<P, float, 0><<<grid, kThreads, smem, s>>>(g, xf, yf, E, bulk_ok); break;
     case 2: k_apply_tile<P, float, 1><<<grid, kThreads, smem, s>>>(g, xf, yf, E, bulk_ok); break;
