@@ -21,13 +21,16 @@ struct EoTable {
   T O[kEoH * (kEoH | 1)], E[kEoH * (kEoH | 1)], C[kEoH], R[kEoH];
 };
 struct EoTables {
-  EoTable<double> D64, H64;        // D and H = Dᵀ W
-  EoTable<float> D32, Dh32, H32;   // D, ½D and H
+  EoTable<double> D64, T64, H64;        // D, Dᵀ and H = Dᵀ W
+  EoTable<float> D32, T32, Dh32, H32;   // the same, and ½D
 };
 static __constant__ EoTables c_eo;
 template <class T> __device__ __forceinline__ const EoTable<T>& eo_D();
 template <> __device__ __forceinline__ const EoTable<double>& eo_D<double>() { return c_eo.D64; }
 template <> __device__ __forceinline__ const EoTable<float>& eo_D<float>() { return c_eo.D32; }
+template <class T> __device__ __forceinline__ const EoTable<T>& eo_T();
+template <> __device__ __forceinline__ const EoTable<double>& eo_T<double>() { return c_eo.T64; }
+template <> __device__ __forceinline__ const EoTable<float>& eo_T<float>() { return c_eo.T32; }
 template <class T> __device__ __forceinline__ const EoTable<T>& eo_H();
 template <> __device__ __forceinline__ const EoTable<double>& eo_H<double>() { return c_eo.H64; }
 template <> __device__ __forceinline__ const EoTable<float>& eo_H<float>() { return c_eo.H32; }

@@ -35,6 +35,7 @@
 
 #include "mesh_index.cuh"
 #include "surface_device.cuh"
+#include "even_odd.cuh"
 
 namespace semgb {
 
@@ -152,15 +153,18 @@ __global__ void k_diag(DevGeom g) {
 // ------------------------------------------------------------------------------------
 template <int P, class T>
 struct Smem {
-  static constexpr int Q = P + 1;
+  static constexpr int Q = P + 1, QP = Q | 1;   // QP: odd stride of the line buffers
   T* D;     // Q*Q
   T* w;     // Q
   T* sig;   // nrow
   T* cxz;   // E*2*Nz: Δσ_l/Δx_e, Δx_e/Δσ_l of the chunk's element columns
   T* geo;   // E*4*Q
   T* X;     // E*Q*nrow
-  T* F1;    // E*Nz*Q*Q
-  T* F2;    // E*Nz*Q*Q
+  T* F1;    // E*Nz*Q*QP
+  T* F2;    // E*Nz*Q*QP
+  T* Y;     // E*nrow*QP
+  T* top;   // E*Nz*Q   contributions to the rows shared with the layer above
+  T* end;
   __device__ void carve(unsigned char* base, int nrow, int Nz, int E) {
     T* p = reinterpret_cast<T*>(base);
     D = p; p += Q * Q;
@@ -169,8 +173,11 @@ struct Smem {
     cxz = p; p += 2 * Nz * E;
     geo = p; p += 4 * Q * E;
     X = p; p += Q * nrow * E;
-    F1 = p; p += Nz * Q * Q * E;
-    F2 = p;
+    F1 = p; p += Nz * Q * QP * E;
+    F2 = p; p += Nz * Q * QP * E;
+    Y = p; p += nrow * QP * E;
+    top = p; p += Nz * Q * E;
+    end = p;
   }
   __device__ void load_tables(const DevGeom& g) {
     const T* cD = CT<T>::D() + d_off(P);
@@ -203,24 +210,33 @@ __device__ __forceinline__ void geo_factors(T d, T invd, T hx, T dxd, T cz0, T c
   G22 = wab * cz1 * K22;
 }
 
-// The factors of every element-local node of the CTA's element columns R.e0..R.e1−1, three per
-// node in the order of the apply's work items; FP64, computed as in apply_element_chunk.
+// The factors of every element-local node of the CTA's element columns R.e0..R.e1−1, FP64, computed as in
+// the applies, in the order that the apply reads: node by node, or (lines) [element, layer][factor][b][a], so
+// that consecutive lanes, at consecutive a, read consecutive words.
 template <int P>
-__device__ void fill_gcache(const DevGeom& g, int e0, int e1, double* gc) {
-  constexpr int Q = P + 1;
-  const int elsz = g.Nz * Q * Q;
+__device__ void fill_gcache(const DevGeom& g, int e0, int e1, double* gc, bool lines) {
+  constexpr int Q = P + 1, QQ = Q * Q;
+  const int elsz = g.Nz * QQ;
   const double* w = c_w64 + w_off(P);
   for (int t = threadIdx.x; t < (e1 - e0) * elsz; t += blockDim.x) {
     const int e = g.dv_elsz.div(t), rem0 = t - e * elsz;
-    const int l = rem0 / (Q * Q), rem = rem0 - l * (Q * Q), a = rem / Q, b = rem - a * Q;
+    const int l = rem0 / QQ, rem = rem0 - l * QQ;
+    const int hi = rem / Q, lo = rem - hi * Q, a = lines ? lo : hi, b = lines ? hi : lo;
     const int ge = e0 + e;
     const double* geo = g.geo64 + (size_t)ge * Q * 4 + a * 4;
     const double* cz = g.cxz + ((size_t)ge * g.Nz + l) * 2;   // the layer's ratios, not a division per node
     double G11, G12, G22;
     geo_factors<double>(geo[0], geo[1], geo[2], geo[3], cz[0], cz[1], w[a], w[b], g.sig[l * P + b], G11, G12, G22);
-    gc[3 * t] = G11;
-    gc[3 * t + 1] = G12;
-    gc[3 * t + 2] = G22;
+    if (lines) {
+      double* o = gc + (size_t)(e * g.Nz + l) * 3 * QQ + rem;
+      o[0] = G11;
+      o[QQ] = G12;
+      o[2 * QQ] = G22;
+    } else {
+      gc[3 * t] = G11;
+      gc[3 * t + 1] = G12;
+      gc[3 * t + 2] = G22;
+    }
   }
 }
 
@@ -281,39 +297,179 @@ __device__ __forceinline__ T apply_element_chunk(const DevGeom& g, Smem<P, T>& s
     s.F2[t] = fmx(G12, ur, G22 * ut);
   }
   __syncthreads();
+  // the transposed sums of every node in its own layer; the rows shared between layers are the lower
+  // row of the upper layer, and the upper row of the lower one goes to s.top (items of their own: as a
+  // second pair of loops inside the first items they made every warp run both)
+  const int ntop = TOP ? 0 : ne * (Nz - 1) * Q, nmain = ne * colsz;
+  for (int t = threadIdx.x; t < nmain + ntop; t += blockDim.x) {
+    int e, l, a, b;
+    T* out;
+    if (t < nmain) {
+      e = g.dv_colsz.div(t);
+      const int rem = t - e * colsz;
+      a = g.dv_nrow.div(rem);
+      const int iz = rem - a * nrow;
+      l = iz / P;
+      b = iz - l * P;
+      if (l == Nz) { l = Nz - 1; b = P; }
+      if (TOP && l < l_first) continue;
+      out = s.Y + t;
+    } else {
+      const int q = t - nmain, el = q / Q;
+      a = q - el * Q;
+      e = Nz == 2 ? el : el / (Nz - 1);
+      l = el - e * (Nz - 1);
+      b = P;
+      out = s.top + (e * Nz + l) * Q + a;
+    }
+    const T* F1 = s.F1 + e * elsz + (l * Q) * Q + b;       // F1[(l*Q+a')*Q+b] = F1[a'*Q]
+    const T* F2 = s.F2 + e * elsz + (l * Q + a) * Q;       // F2[(l*Q+a)*Q+b']
+    T y = 0;
+#pragma unroll
+    for (int c = 0; c < Q; ++c) {
+      y = fmx(s.D[c * Q + a], F1[c * Q], y);
+      y = fmx(s.D[c * Q + b], F2[c], y);
+    }
+    *out = y;
+  }
+  __syncthreads();
   T part = 0;
   for (int t = threadIdx.x; t < ne * colsz; t += blockDim.x) {
     const int e = g.dv_colsz.div(t), rem = t - e * colsz;
     const int a = g.dv_nrow.div(rem), iz = rem - a * nrow;
-    const int l = iz / P, b = iz - l * P;
+    const int l = iz / P;
     if (TOP && l < l_first) continue;
-    const T* F1e = s.F1 + e * elsz;
-    const T* F2e = s.F2 + e * elsz;
-    T y = 0;
-    if (l < Nz) {
-      const T* F1 = F1e + (l * Q) * Q + b;       // F1[(l*Q+a')*Q+b] = F1[a'*Q]
-      const T* F2 = F2e + (l * Q + a) * Q;       // F2[(l*Q+a)*Q+b']
-#pragma unroll
-      for (int c = 0; c < Q; ++c) {
-        y = fmx(s.D[c * Q + a], F1[c * Q], y);
-        y = fmx(s.D[c * Q + b], F2[c], y);
-      }
-    }
-    if (b == 0 && l > l_first) {
-      const int lm = l - 1;
-      const T* F1 = F1e + (lm * Q) * Q + P;
-      const T* F2 = F2e + (lm * Q + a) * Q;
-#pragma unroll
-      for (int c = 0; c < Q; ++c) {
-        y = fmx(s.D[c * Q + a], F1[c * Q], y);
-        y = fmx(s.D[c * Q + P], F2[c], y);
-      }
-    }
+    T y = s.Y[t];
+    if (!TOP && iz - l * P == 0 && l > 0 && l < Nz) y += s.top[(e * Nz + l - 1) * Q + a];
     store(ex0 + e, a, iz, y);
     part = fmx(s.X[t], y, part);
   }
   __syncthreads();
   return part;
+}
+
+// The same apply by lines in registers with the even-odd forms of D and Dᵀ (even_odd.cuh), for chunks with
+// enough lines to keep every SM sub-partition busy: about 25 FP64 operations per node (P = 6) instead of
+// 33 of the node-by-node form, each of which holds the narrow FP64 pipe for a whole warp's time.
+//   x-lines (element, row): u_r;  σ-lines (element, layer, column): u_t, the fluxes F1, F2 and the σ part of the
+//   transposed sum;  x-lines: the x part, over the rows of the whole column (F1 of a row shared by two
+//   layers is added up first), and the stores (consecutive lanes: consecutive rows of a column).
+// gc: factors in the line order of fill_gcache, or nullptr (the geometry is staged and they are computed).
+// An FP64 apply of the 512 uneven tanks takes 55 instead of 59 µs of a tank's team, an FP32 one 12.5
+// instead of 15.8 (step 12.17 → 11.85 and 11.31 → 10.89 ms), one of the 2048×2 shoal 16.6 instead of 17.9.
+// Shorter chunks (under kLineMin σ-lines, less than one warp per sub-partition: 64×4 elements on 64 CTAs)
+// keep the node-by-node form, 4.0 µs where one warp of lines would take about 6 (4.3 before its shared
+// rows became items of their own).
+constexpr int kLineMin = 112, kLineMaxP = 9;
+template <int P>
+__device__ __forceinline__ bool use_lines(const DevGeom& g, int ne) {
+  return P <= kLineMaxP && min(g.chunk, ne) * g.Nz * (P + 1) >= kLineMin;
+}
+
+template <int P, class T, class LoadX, class Store>
+__device__ __forceinline__ T apply_element_lines(const DevGeom& g, Smem<P, T>& s, int ex0, int ne, LoadX loadx,
+                                                 Store store, const double* gc = nullptr) {
+  constexpr int Q = P + 1, QP = Smem<P, T>::QP, QQ = Q * Q;
+  const int nrow = g.nrow, Nz = g.Nz, colsz = Q * nrow;
+  if (gc == nullptr) {
+    const T* geo = geo_ptr<T>(g) + (size_t)ex0 * Q * 4;
+    for (int t = threadIdx.x; t < ne * 4 * Q; t += blockDim.x) s.geo[t] = geo[t];
+    const double* cz = g.cxz + (size_t)ex0 * Nz * 2;
+    for (int t = threadIdx.x; t < ne * Nz * 2; t += blockDim.x) s.cxz[t] = (T)cz[t];
+  }
+  for (int t = threadIdx.x; t < ne * colsz; t += blockDim.x) {
+    const int e = g.dv_colsz.div(t), rem = t - e * colsz;
+    const int a = g.dv_nrow.div(rem), iz = rem - a * nrow;
+    s.X[t] = loadx(ex0 + e, a, iz);
+  }
+  __syncthreads();
+#pragma unroll 1
+  for (int t = threadIdx.x; t < ne * nrow; t += blockDim.x) {
+    const int e = g.dv_nrow.div(t), iz = t - e * nrow;
+    const T* x = s.X + e * colsz + iz;
+    T u[Q], r[Q];
+#pragma unroll
+    for (int c = 0; c < Q; ++c) u[c] = x[c * nrow];
+    eo_line<Q, T>(eo_D<T>(), u, r);
+#pragma unroll
+    for (int a = 0; a < Q; ++a) s.Y[t * QP + a] = r[a];
+  }
+  __syncthreads();
+#pragma unroll 1
+  for (int t = threadIdx.x; t < ne * Nz * Q; t += blockDim.x) {
+    const int el = t / Q, a = t - el * Q;
+    const int e = Nz == 1 ? el : el / Nz, l = el - e * Nz;
+    const T* x = s.X + e * colsz + a * nrow + l * P;
+    const T* ur = s.Y + (e * nrow + l * P) * QP + a;
+    T u[Q], ut[Q], f[Q];
+#pragma unroll
+    for (int c = 0; c < Q; ++c) u[c] = x[c];
+    eo_line<Q, T>(eo_D<T>(), u, ut);
+    const double* gl = gc ? gc + (size_t)el * 3 * QQ + a : nullptr;
+    T* F = s.F1 + (size_t)el * Q * QP + a;
+#pragma unroll
+    for (int b = 0; b < Q; ++b) {
+      T G11, G12, G22;
+      if (gl) {
+        G11 = (T)gl[b * Q];
+        G12 = (T)gl[QQ + b * Q];
+        G22 = (T)gl[2 * QQ + b * Q];
+      } else {
+        const T* ge = s.geo + e * 4 * Q + a * 4;
+        geo_factors<T>(ge[0], ge[1], ge[2], ge[3], s.cxz[2 * el], s.cxz[2 * el + 1], s.w[a], s.w[b], s.sig[l * P + b],
+                       G11, G12, G22);
+      }
+      const T r = ur[b * QP];
+      F[b * QP] = fmx(G11, r, G12 * ut[b]);
+      f[b] = fmx(G12, r, G22 * ut[b]);
+    }
+    eo_line<Q, T>(eo_T<T>(), f, ut);
+    T* ys = s.F2 + (size_t)el * Q * QP + a;
+#pragma unroll
+    for (int b = 0; b < Q; ++b) ys[b * QP] = ut[b];
+  }
+  __syncthreads();
+  T part = 0;
+#pragma unroll 1
+  for (int t = threadIdx.x; t < ne * nrow; t += blockDim.x) {
+    const int e = g.dv_nrow.div(t), iz = t - e * nrow;
+    int l = iz / P, b = iz - l * P;
+    if (l == Nz) { l = Nz - 1; b = P; }
+    const bool shared = b == 0 && l > 0;             // row P of the layer below is the same row
+    const int at = ((e * Nz + l) * Q + b) * QP, lo = ((e * Nz + l - 1) * Q + P) * QP;
+    T f[Q], y[Q];
+#pragma unroll
+    for (int c = 0; c < Q; ++c) f[c] = s.F1[at + c];
+    if (shared) {
+#pragma unroll
+      for (int c = 0; c < Q; ++c) f[c] += s.F1[lo + c];
+    }
+    eo_line<Q, T>(eo_T<T>(), f, y);
+#pragma unroll
+    for (int a = 0; a < Q; ++a) y[a] += s.F2[at + a];
+    if (shared) {
+#pragma unroll
+      for (int a = 0; a < Q; ++a) y[a] += s.F2[lo + a];
+    }
+    const T* x = s.X + e * colsz + iz;
+#pragma unroll
+    for (int a = 0; a < Q; ++a) {
+      store(ex0 + e, a, iz, y[a]);
+      part = fmx(x[a * nrow], y[a], part);
+    }
+  }
+  __syncthreads();
+  return part;
+}
+
+// One of the two, by the team's `lines` (use_lines; the order of gc follows it).
+template <int P, class T, class LoadX, class Store>
+__device__ __forceinline__ T apply_elements(const DevGeom& g, Smem<P, T>& s, int ex0, int ne, LoadX loadx, Store store,
+                                            const double* gc, bool lines) {
+  if constexpr (P <= kLineMaxP) {
+    if (lines) return apply_element_lines<P, T>(g, s, ex0, ne, loadx, store, gc);
+  }
+  return apply_element_chunk<P, T>(g, s, ex0, ne, loadx, store, gc);
 }
 
 // ------------------------------------------------------------------------------------
@@ -344,7 +500,6 @@ __global__ void __launch_bounds__(kThreads) k_apply(DevGeom g, const double* __r
 
 }  // namespace semgb
 
-#include "even_odd.cuh"
 #include "apply_tile.cuh"
 #include "apply_elem.cuh"
 #include "apply_tc.cuh"
@@ -845,6 +1000,7 @@ __device__ int cg_solve(const DevGeom& g, Smem<P, T>& s, const Range& R, const T
   __shared__ T s_scal[2];
   __shared__ int s_stop;
   int cur = 0;
+  const bool lines = use_lines<P>(g, R.e1 - R.e0);
   SEM_MARK(g, tm, TR_CG_START);
   cg_update<P, T, TP, CACHE>(g, s, R, tm, pv, PA.precond, V, cur, false, true, T(0), T(0));
   if (!finish_precondition<P, T, TP, CACHE>(g, s, R, tm, PA, pv, V, s_flag)) return -1;
@@ -860,7 +1016,7 @@ __device__ int cg_solve(const DevGeom& g, Smem<P, T>& s, const Range& R, const T
     A acc[3] = {A(0), A(0), A(0)};   // γ = (r,u), δ = (u,Au), (r,r)
     for (int ex0 = R.e0; ex0 < R.e1; ex0 += g.chunk) {
       const double* gce = gc ? gc + (size_t)(ex0 - R.e0) * 3 * g.Nz * (P + 1) * (P + 1) : nullptr;
-      acc[1] += (A)apply_element_chunk<P, T>(
+      acc[1] += (A)apply_elements<P, T>(
           g, s, ex0, min(g.chunk, R.e1 - ex0),
           [&](int e, int a, int iz) -> T {
             if (iz == nrow - 1) return T(0);
@@ -878,7 +1034,7 @@ __device__ int cg_solve(const DevGeom& g, Smem<P, T>& s, const Range& R, const T
             if (owns_local_col(g, e, a)) V.w[(size_t)col_of(g, e, a) * nrow + iz] = y;
             else V.edge[(size_t)e * nrow + iz] = y;
           },
-          gce);
+          gce, lines);
     }
     block_sum<3, A>(acc, red);
     put_partials<3, A>(tm, 2, acc);
@@ -945,11 +1101,12 @@ __device__ bool fp64_residual(const DevGeom& g, Smem<P, double>& s, const Range&
   const int nrow = g.nrow;
   const double* x = A.x;
   const double* phis = A.phis;
+  const bool lines = use_lines<P>(g, R.e1 - R.e0);
   const size_t gstride = (size_t)3 * g.Nz * (g.P + 1) * (g.P + 1);   // cached factors per element
   for (int ex0 = R.e0; ex0 < R.e1; ex0 += g.chunk) {
     const int ne = min(g.chunk, R.e1 - ex0);
     const double* gce = gc ? gc + (size_t)(ex0 - R.e0) * gstride : nullptr;
-    apply_element_chunk<P, double>(
+    apply_elements<P, double>(
         g, s, ex0, ne,
         [&](int e, int a, int iz) -> double {
           const int col = col_of(g, e, a);
@@ -961,7 +1118,7 @@ __device__ bool fp64_residual(const DevGeom& g, Smem<P, double>& s, const Range&
           if (owns_local_col(g, e, a)) A.q64[(size_t)col_of(g, e, a) * nrow + iz] = y;
           else A.edge64[(size_t)e * nrow + iz] = y;
         },
-        gce);
+        gce, lines);
   }
   if (want_b) {
     // b = −(A[0; φ̃])_I enters only through ‖b‖, the scale of the stopping test, which FP32 gives to
@@ -1042,16 +1199,17 @@ __device__ bool solve_body(const DevGeom& g, const PcgArgs& A, const Team& tm, u
   // the geometric factors of the FP64 applies, once per solve, where the launch reserved room
   // for them after the apply's buffers
   // (in shared memory where the launch reserved room, else in the mesh's global array)
+  const bool lines = use_lines<P>(g, R.e1 - R.e0);
   const double* gc = nullptr;
   const size_t per_e = (size_t)3 * g.Nz * (P + 1) * (P + 1);
   if (g.gcache > 0 && per_e * (R.e1 - R.e0) <= (size_t)g.gcache) {
-    double* c = s64.F2 + (size_t)g.Nz * (P + 1) * (P + 1) * g.chunk;
-    fill_gcache<P>(g, R.e0, R.e1, c);
+    double* c = s64.end;
+    fill_gcache<P>(g, R.e0, R.e1, c, lines);
     __syncthreads();
     gc = c;
   } else if (g.gglob != nullptr) {
     double* c = g.gglob + (size_t)R.e0 * per_e;
-    fill_gcache<P>(g, R.e0, R.e1, c);
+    fill_gcache<P>(g, R.e0, R.e1, c, lines);
     __syncthreads();
     gc = c;
   }
@@ -1526,7 +1684,8 @@ __device__ void stage_body(Instance& I, const Team& tm, int stage, int step, uns
   {
     double* kxs = reinterpret_cast<double*>(smem_raw);
     constexpr int per = Q * Q + Q;
-    const int avail = Q * Q + Q + g.nrow + g.chunk * (2 * g.Nz + 4 * Q + Q * g.nrow + 2 * g.Nz * Q * Q);
+    const int avail = Q * Q + Q + g.nrow +
+                      g.chunk * (2 * g.Nz + 4 * Q + Q * g.nrow + g.nrow * (Q | 1) + 2 * g.Nz * Q * (Q | 1) + g.Nz * Q);
     const int nb_max = max(1, min(ne, avail / per));
     const int nr = I.ps.nr;
     for (int e0 = R.e0; e0 < R.e1; e0 += nb_max) {
@@ -1693,11 +1852,16 @@ cudaError_t upload_tables_impl(const double* D64, const double* w64) {
   constexpr int Q = P + 1;
   const double* D = D64 + d_off(P);
   const double* w = w64 + w_off(P);
-  double H[Q * Q];
+  double H[Q * Q], Dt[Q * Q];
   for (int i = 0; i < Q; ++i)
-    for (int j = 0; j < Q; ++j) H[i * Q + j] = D[j * Q + i] * w[j];
+    for (int j = 0; j < Q; ++j) {
+      Dt[i * Q + j] = D[j * Q + i];
+      H[i * Q + j] = D[j * Q + i] * w[j];
+    }
   EoTables eo{};
   fill_eo<P>(eo.D64, D, 1.0);
+  fill_eo<P>(eo.T64, Dt, 1.0);
+  fill_eo<P>(eo.T32, Dt, 1.0);
   fill_eo<P>(eo.H64, H, 1.0);
   fill_eo<P>(eo.D32, D, 1.0);
   fill_eo<P>(eo.Dh32, D, 0.5);
