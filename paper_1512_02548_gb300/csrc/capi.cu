@@ -172,11 +172,7 @@ struct sem_mesh {
   double* wkx = nullptr;
   double hist_dt = 0.0;
   const double *hist_eta = nullptr, *hist_phis = nullptr;
-  // fused-stage launch of this mesh alone: device descriptor, CTA map, barrier pair
-  Instance* inst_d = nullptr;
-  int* cta_inst_d = nullptr;
-  unsigned int* stage_bars = nullptr;
-  Instance inst_h{};
+  unsigned int* stage_bars = nullptr;   // barrier pair of this mesh's own fused stage launch
   int stage_team = 0;
   size_t stage_smem = 0;         // the mesh's own fused stage launch (with the factor cache)
   size_t stage_smem_batch = 0;   // in a batch launch (no factor cache)
@@ -281,7 +277,11 @@ int do_solve(sem_mesh* m, const double* phis, double* Phi, cudaStream_t s) {
     CUDA_TRY(take_event(m, &e1));
     CUDA_TRY(cudaEventRecord(e0, s));
   }
-  CUDA_TRY(launch_pcg(m->g, a, m->grid, m->smem, s));
+  // the shape of the mesh's own fused stage launch: one pass over a CTA's columns, the factor cache
+  DevGeom g = m->g;
+  g.chunk = m->own_chunk;
+  g.gcache = m->gcache;
+  CUDA_TRY(launch_pcg(g, a, m->stage_team, m->stage_smem, s));
   if (m->timing) {
     CUDA_TRY(cudaEventRecord(e1, s));
     m->events.emplace_back(e0, e1);
@@ -298,9 +298,20 @@ int do_geometry(sem_mesh* m, const double* eta, cudaStream_t s) {
 
 bool has_zones(const sem_mesh* m) { return m->p.relax_left > 0.0 || m->p.relax_right > 0.0; }
 
+int launch_own_stage(sem_mesh* m, const StageArgs& a, cudaStream_t s);
+Instance make_instance(sem_mesh* m, double* eta, double* phis, double tstart, double dt, int team0, int nteam,
+                       bool own_launch = false, int chunk = 0);
+
 int do_rhs(sem_mesh* m, const double* eta, const double* phis, double time, double tau, double* de,
            double* dp, cudaStream_t s) {
-  const int Q = m->p.P + 1;
+  if (m->fused) {   // the fused stage without its RK4 update: one launch instead of seven
+    StageArgs a{nullptr, nullptr, m->stage_bars, 5, 0, 0,
+                make_instance(m, const_cast<double*>(eta), const_cast<double*>(phis), time, 1.0, 0, m->stage_team, true)};
+    a.own.ke = de;
+    a.own.kp = dp;
+    a.own.tau = tau;
+    return launch_own_stage(m, a, s);
+  }
   int rc0 = do_geometry(m, eta, s);
   if (rc0) return rc0;
   int rc = do_solve(m, phis, m->Phi, s);
@@ -309,7 +320,6 @@ int do_rhs(sem_mesh* m, const double* eta, const double* phis, double time, doub
   CUDA_TRY(launch_zakharov(m->st, eta, m->etax, m->phisx, m->wt, m->R, s));
   CUDA_TRY(launch_mass1d(m->st, m->R, de, dp, s));
   if (has_zones(m)) CUDA_TRY(launch_relax(m->st, eta, phis, time, 1.0 / tau, de, dp, s));
-  (void)Q;
   return SEM_OK;
 }
 
@@ -325,7 +335,7 @@ void set_history(sem_mesh* m, const double* eta, const double* phis, double dt) 
 // own_launch: the mesh's own fused stage launch, whose shared memory holds the factor cache.
 // chunk > 0: element columns per pass in a batch launch.
 Instance make_instance(sem_mesh* m, double* eta, double* phis, double tstart, double dt, int team0,
-                       int nteam, bool own_launch = false, int chunk = 0) {
+                       int nteam, bool own_launch, int chunk) {
   Instance I{};
   I.g = m->g;
   I.g.gcache = own_launch ? m->gcache : 0;
@@ -348,28 +358,31 @@ Instance make_instance(sem_mesh* m, double* eta, double* phis, double tstart, do
   return I;
 }
 
+// One fused stage launch of a mesh alone (a.own filled in).
+int launch_own_stage(sem_mesh* m, const StageArgs& a, cudaStream_t s) {
+  cudaEvent_t e0 = nullptr, e1 = nullptr;
+  if (m->timing) {
+    CUDA_TRY(take_event(m, &e0));
+    CUDA_TRY(take_event(m, &e1));
+    CUDA_TRY(cudaEventRecord(e0, s));
+  }
+  CUDA_TRY(launch_stage(m->p.P, m->p.precision == SEM_PREC_MIXED, 0, a, m->stage_team, m->stage_smem, s));
+  if (m->timing) {
+    CUDA_TRY(cudaEventRecord(e1, s));
+    m->events.emplace_back(e0, e1);
+  }
+  return SEM_OK;
+}
+
 // nsteps RK4 steps of one mesh with the fused stage kernel: one cooperative launch per stage.
 int do_rk4_fused(sem_mesh* m, double* eta, double* phis, double t0, double dt, int nsteps, cudaStream_t s) {
-  m->inst_h = make_instance(m, eta, phis, t0, dt, 0, m->stage_team, true);
-  CUDA_TRY(cudaMemcpyAsync(m->inst_d, &m->inst_h, sizeof(Instance), cudaMemcpyHostToDevice, s));
-  StageArgs a{m->inst_d, m->cta_inst_d, m->stage_bars, 1, 0, 0};
-  const int mixed = m->p.precision == SEM_PREC_MIXED;
+  StageArgs a{nullptr, nullptr, m->stage_bars, 1, 0, 0, make_instance(m, eta, phis, t0, dt, 0, m->stage_team, true)};
   for (int step = 0; step < nsteps; ++step)
     for (int stage = 1; stage <= 4; ++stage) {
       a.stage = stage;
       a.step = step;
-      CUDA_TRY(cudaMemsetAsync(m->stage_bars, 0, 2 * sizeof(unsigned int), s));
-      cudaEvent_t e0 = nullptr, e1 = nullptr;
-      if (m->timing) {
-        CUDA_TRY(take_event(m, &e0));
-        CUDA_TRY(take_event(m, &e1));
-        CUDA_TRY(cudaEventRecord(e0, s));
-      }
-      CUDA_TRY(launch_stage(m->p.P, mixed, 0, a, m->stage_team, m->stage_smem, s));
-      if (m->timing) {
-        CUDA_TRY(cudaEventRecord(e1, s));
-        m->events.emplace_back(e0, e1);
-      }
+      const int rc = launch_own_stage(m, a, s);
+      if (rc) return rc;
     }
   if (nsteps > 0) set_history(m, eta, phis, dt);
   return SEM_OK;
@@ -707,7 +720,7 @@ static int mesh_create_impl(const sem_params* pin, const double* x_edges_h, cons
                o_P1 = cv.take<double>(n), o_P2 = cv.take<double>(n), o_P3 = cv.take<double>(n),
                o_D32 = cv.take<double>(n);
   const size_t o_gglob = cv.take<double>((size_t)3 * Nx * Nz * Q * Q);
-  const size_t o_inst = cv.take<Instance>(1), o_ctai = cv.take<int>((size_t)m->grid), o_sbar = cv.take<unsigned>(4);
+  const size_t o_sbar = cv.take<unsigned>(4);
   const size_t total = cv.off + 256;
   if (footprint_only) {
     *footprint_only = total;
@@ -818,8 +831,6 @@ static int mesh_create_impl(const sem_params* pin, const double* x_edges_h, cons
   m->eta_dev = D_(o_etad); m->phis_dev = D_(o_phisd);
   m->s1e = D_(o_s1e); m->s1p = D_(o_s1p);
   m->Phi1 = D_(o_P1); m->Phi2 = D_(o_P2); m->Phi3 = D_(o_P3); m->D32 = D_(o_D32);
-  m->inst_d = reinterpret_cast<Instance*>(m->pool + o_inst);
-  m->cta_inst_d = reinterpret_cast<int*>(m->pool + o_ctai);
   m->stage_bars = reinterpret_cast<unsigned int*>(m->pool + o_sbar);
 
   SurfTables& t = m->st;
@@ -870,13 +881,6 @@ static int mesh_create_impl(const sem_params* pin, const double* x_edges_h, cons
         m->stage_smem = smem2;
         m->gcache = (int)need;
       }
-    }
-    std::vector<int> zeros(m->grid, 0);
-    cudaError_t e2 = cudaMemcpy(m->cta_inst_d, zeros.data(), sizeof(int) * m->grid, cudaMemcpyHostToDevice);
-    if (e2 != cudaSuccess) {
-      dev_free(dev, m->pool);
-      delete m;
-      return fail(SEM_ERR_CUDA, std::string("upload: ") + cudaGetErrorString(e2));
     }
   }
   *out = m;
@@ -1510,7 +1514,7 @@ cudaError_t run_clusters(sem_batch* b, int stage, int nsteps, cudaStream_t s) {
   for (int step = 0; step < (stage == 0 ? 1 : nsteps); ++step)
     for (int st = (stage == 0 ? 0 : 1); st <= (stage == 0 ? 0 : 4); ++st)
       for (auto& L : b->cl_launches) {
-        const StageArgs a{L.inst_d, L.cta_d, nullptr, st, step, 1};
+        const StageArgs a{L.inst_d, L.cta_d, nullptr, st, step, 1, {}};
         if ((e = batch_launch(b, L, a, L.stream)) != cudaSuccess) return e;
       }
   for (auto& L : b->cl_launches) {
@@ -1549,7 +1553,7 @@ int sem_batch_rk4_step(sem_batch* b, double* const* eta_d, double* const* phis_d
       for (int stage = 1; stage <= 4; ++stage)
         for (auto& L : plan) {
           CUDA_TRY(cudaMemsetAsync(L.bars_d, 0, 2 * sizeof(unsigned int) * L.members.size(), s));
-          const StageArgs a{L.inst_d, L.cta_d, L.bars_d, stage, step, 0};
+          const StageArgs a{L.inst_d, L.cta_d, L.bars_d, stage, step, 0, {}};
           CUDA_TRY(batch_launch(b, L, a, s));
         }
   }
@@ -1586,7 +1590,7 @@ int sem_batch_laplace_solve(sem_batch* b, const double* const* eta_d, const doub
   } else {
     for (auto& L : plan) {
       CUDA_TRY(cudaMemsetAsync(L.bars_d, 0, 2 * sizeof(unsigned int) * L.members.size(), s));
-      const StageArgs a{L.inst_d, L.cta_d, L.bars_d, 0, 0, 0};
+      const StageArgs a{L.inst_d, L.cta_d, L.bars_d, 0, 0, 0, {}};
       CUDA_TRY(batch_launch(b, L, a, s));
     }
   }

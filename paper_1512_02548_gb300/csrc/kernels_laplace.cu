@@ -269,8 +269,7 @@ cudaError_t launch_prec_setup(const DevGeom& g, const PrecSetup& ps, cudaStream_
 }
 
 cudaError_t launch_pcg(const DevGeom& g, const PcgArgs& a, int grid, size_t smem, cudaStream_t s) {
-  cudaError_t e = cudaMemsetAsync(a.bar, 0, 2 * sizeof(unsigned int), s);
-  if (e != cudaSuccess) return e;
+  cudaError_t e = cudaSuccess;
   SEM_DISPATCH_P(g.P, (e = launch_pcg_impl<PP>(a.mixed, g, a, grid, smem, s)));
   count_launch();
   return e;

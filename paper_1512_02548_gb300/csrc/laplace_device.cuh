@@ -592,6 +592,15 @@ static __device__ __forceinline__ bool grid_barrier(const Team& tm, int* s_flag)
   return *s_flag != 0;
 }
 
+// The CTA's last act in a launch whose team barrier is the global one: the last CTA to leave (the exit
+// counter wraps to zero by itself) zeroes the arrival counter for the next launch.  Every CTA calls it on
+// every way out, after its last poll.
+static __device__ __forceinline__ void bar_leave(const Team& tm) {
+  if (tm.cluster || tm.size == 1) return;
+  __syncthreads();
+  if (threadIdx.x == 0 && atomicInc(tm.bar + 1, (unsigned)tm.size - 1) == (unsigned)tm.size - 1) atomicExch(tm.bar, 0u);
+}
+
 // Shared reduction buffer of the persistent kernels: K·blockDim partials of block_sum, then the
 // block sums and the grid sums.
 constexpr int kRedOut = 4 * kThreads, kRedGrid = kRedOut + 8, kRedSize = kRedGrid + 8;
@@ -1315,15 +1324,18 @@ __device__ bool solve_body(const DevGeom& g, const PcgArgs& A, const Team& tm, u
   return true;
 }
 
+// One CTA per SM with the full register file, like the mesh's own fused stage launch, with the same chunks
+// and factor cache.
 template <int P, bool MIXED>
-__global__ void __launch_bounds__(kThreads) k_pcg(DevGeom g, PcgArgs A) {
+__global__ void __launch_bounds__(kThreads, 1) k_pcg(DevGeom g, PcgArgs A) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double red[kRedSize];
   __shared__ int s_flag[2];   // barrier result, barriers passed
   if (threadIdx.x == 0) s_flag[1] = 0;
   const Team tm{(int)blockIdx.x, (int)gridDim.x, A.bar, g.status, A.part, A.part_stride, g.bar_timeout_ns, 0};
-  if (tm.rank == g.drop_rank) return;   // testing hook: see sem_set_barrier_test
-  solve_body<P, MIXED>(g, A, tm, smem_raw, red, s_flag);
+  // testing hook: see sem_set_barrier_test
+  if (tm.rank != g.drop_rank) solve_body<P, MIXED, true>(g, A, tm, smem_raw, red, s_flag);
+  bar_leave(tm);
 }
 
 // ------------------------------------------------------------------------------------
@@ -1647,8 +1659,14 @@ static __device__ void prec_tri_mode_cta(const DevGeom& g, const PrecSetup& ps, 
   }
 }
 
-static __global__ void __launch_bounds__(32) k_prec_tri(DevGeom g, PrecSetup ps, int staged) {
+// A CTA per mode: one warp, or all its warps for long systems between walls (whole = 1; as in the fused
+// stage: 2778 unknowns 228 → 10 µs).
+static __global__ void __launch_bounds__(kThreads) k_prec_tri(DevGeom g, PrecSetup ps, int staged, int whole) {
   extern __shared__ __align__(16) double tri_sm[];
+  if (whole) {
+    prec_tri_mode_cta(g, ps, blockIdx.x);
+    return;
+  }
   prec_tri_mode(g, ps, blockIdx.x, staged ? reinterpret_cast<float*>(tri_sm) : nullptr);
 }
 
@@ -1669,13 +1687,15 @@ __device__ void stage_body(Instance& I, const Team& tm, int stage, int step, uns
   const SurfTables& t = I.st;
   const Range R = my_range(g, tm);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  // stage 0: Laplace solve only (geometry, preconditioner and solve from the state itself)
-  const double* ein = stage <= 1 ? I.eta : (stage == 3 ? I.s1e : I.s0e);
-  const double* pin = stage <= 1 ? I.phis : (stage == 3 ? I.s1p : I.s0p);
+  // stage 0: Laplace solve only (geometry, preconditioner and solve from the state itself); stage 5: the
+  // right-hand side alone, from the state, started from the mesh's last potential
+  const bool from_state = stage <= 1 || stage == 5;
+  const double* ein = from_state ? I.eta : (stage == 3 ? I.s1e : I.s0e);
+  const double* pin = from_state ? I.phis : (stage == 3 ? I.s1p : I.s0p);
   double* eout = stage == 2 ? I.s1e : I.s0e;   // stage inputs of the next stage (not used at stage 4)
   double* pout = stage == 2 ? I.s1p : I.s0p;
   const double t0 = I.tstart + step * I.dt;
-  const double time = t0 + (stage == 1 ? 0.0 : (stage == 4 ? I.dt : 0.5 * I.dt));
+  const double time = t0 + (from_state ? 0.0 : (stage == 4 ? I.dt : 0.5 * I.dt));
   const int ne = R.e1 - R.e0, nc = R.c1 - R.c0;
   SEM_MARK(g, tm, TR_START);
 
@@ -1821,7 +1841,7 @@ __device__ void stage_body(Instance& I, const Team& tm, int stage, int step, uns
   // relaxation source and the RK4 bookkeeping on owned columns
   for (int col = R.c0 + threadIdx.x; col < R.c1; col += blockDim.x) {
     if (I.relax) relax_column(t, ein, pin, time, 1.0 / I.tau, I.ke, I.kp, col, wave_tab ? t.wEP : nullptr);
-    rk4_item(stage, I.dt, I.eta, I.phis, I.ke, I.kp, I.ae, I.ap, eout, pout, col);
+    if (stage != 5) rk4_item(stage, I.dt, I.eta, I.phis, I.ke, I.kp, I.ae, I.ap, eout, pout, col);
   }
   SEM_MARK(g, tm, TR_RK4);
   if (stage == 4 && t.filter_on) {
@@ -1841,16 +1861,16 @@ __device__ void stage_body(Instance& I, const Team& tm, int stage, int step, uns
 // launches of other groups may run at the same time.  Every CTA of a cluster takes the same
 // sequence of barriers: no control path leaves the kernel early in one CTA only.
 template <int P, bool MIXED, bool WIDE>
-__global__ void __launch_bounds__(kThreads, WIDE ? 2 : 1) k_stage(StageArgs B) {
+__global__ void __launch_bounds__(kThreads, WIDE ? 2 : 1) k_stage(const __grid_constant__ StageArgs B) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double red[kRedSize];
   __shared__ int s_flag[2];   // barrier result, barriers passed
   __shared__ __align__(16) double sh[kStageWarps][kSurfScratch];
   __shared__ __align__(16) Instance I;
   if (threadIdx.x == 0) s_flag[1] = 0;
-  const int ii = B.cta_inst[blockIdx.x];
+  const int ii = B.inst ? B.cta_inst[blockIdx.x] : 0;
   {
-    const unsigned int* src = reinterpret_cast<const unsigned int*>(B.inst + ii);
+    const unsigned int* src = reinterpret_cast<const unsigned int*>(B.inst ? B.inst + ii : &B.own);
     unsigned int* dst = reinterpret_cast<unsigned int*>(&I);
     for (int q = threadIdx.x; q < (int)(sizeof(Instance) / 4); q += blockDim.x) dst[q] = src[q];
   }
@@ -1858,8 +1878,9 @@ __global__ void __launch_bounds__(kThreads, WIDE ? 2 : 1) k_stage(StageArgs B) {
   const Team tm{(int)blockIdx.x - I.team0, I.nteam, B.bars + 2 * ii, I.g.status, I.pa.part, I.pa.part_stride,
                 I.g.bar_timeout_ns, B.cluster};
   // testing hook (see sem_set_barrier_test); the cluster plan never serves a mesh that carries it
-  if (!B.cluster && tm.rank == I.g.drop_rank) return;
-  stage_body<P, MIXED, !WIDE>(I, tm, B.stage, B.step, smem_raw, red, s_flag, sh);
+  if (B.cluster || tm.rank != I.g.drop_rank)
+    stage_body<P, MIXED, !WIDE>(I, tm, B.stage, B.step, smem_raw, red, s_flag, sh);
+  bar_leave(tm);
 }
 
 // ------------------------------------------------------------------------------------
@@ -1945,12 +1966,13 @@ cudaError_t launch_prec_setup_impl(const DevGeom& g, const PrecSetup& ps, cudaSt
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const size_t bytes = (size_t)2 * ps.nif * sizeof(float);
-  const int staged = bytes <= kTriStageMax ? 1 : 0;
+  const int whole = ps.nif > 32 * kTridiagRegs && !g.periodic ? 1 : 0;
+  const int staged = !whole && bytes <= kTriStageMax ? 1 : 0;
   if (staged) {
     e = cudaFuncSetAttribute(k_prec_tri, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTriStageMax);
     if (e != cudaSuccess) return e;
   }
-  k_prec_tri<<<ps.nr, 32, staged ? bytes : 0, s>>>(g, ps, staged);
+  k_prec_tri<<<ps.nr, whole ? kThreads : 32, staged ? bytes : 0, s>>>(g, ps, staged, whole);
   count_launch();
   return cudaGetLastError();
 }

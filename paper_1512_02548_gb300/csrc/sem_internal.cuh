@@ -139,7 +139,7 @@ struct PcgArgs {
   float *d32, *r32, *z32, *p32a, *p32b, *q32, *edge32;
   double* part;           // reduction partials [4 slots][4 values][max grid]
   int part_stride;        // max grid
-  unsigned int* bar;      // grid barrier: arrival counter (two words), zero at launch
+  unsigned int* bar;      // grid barrier: arrivals, exits; left at zero by every launch
   SolveRecord* rec;
   double* r64b;           // second residual buffer (double-buffered update)
   float* r32b;
@@ -212,13 +212,15 @@ struct Instance {
 };
 
 struct StageArgs {
-  const Instance* inst;  // device array
+  const Instance* inst;  // device array; nullptr: the one instance `own`
   const int* cta_inst;   // CTA → instance
-  unsigned int* bars;    // 2 per instance, zero at launch (cooperative launches)
-  int stage;             // 1..4; 0 = Laplace solve only
+  unsigned int* bars;    // 2 per instance (arrivals, exits), left at zero by every launch (cooperative launches)
+  int stage;             // 1..4; 0 = Laplace solve only; 5 = right-hand side only (I.ke, I.kp)
   int step;              // steps since tstart
   int cluster;           // 1: cluster-team launch (each instance's CTAs are one cluster)
+  Instance own;          // a mesh's own launch: its descriptor travels with the launch, no copy before it
 };
+static_assert(sizeof(StageArgs) <= 4096, "kernel parameters");
 
 // ---- per-order entry points (laplace_device.cuh, instantiated in kernels_order.cu) ----
 template <int P> cudaError_t upload_tables_impl(const double* D64, const double* w64);
