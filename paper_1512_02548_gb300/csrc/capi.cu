@@ -163,15 +163,15 @@ struct sem_mesh {
   double *ke = nullptr, *kp = nullptr, *ae = nullptr, *ap = nullptr, *se = nullptr, *sp = nullptr;
   double *eta_dev = nullptr, *phis_dev = nullptr;
   double *s1e = nullptr, *s1p = nullptr;   // second stage-input pair of the fused RK stage
-  // stage potentials kept for the next stages' initial guesses, and the trajectory they belong
-  // to (the state buffers and dt of the last fused RK call; hist_dt = 0: none)
-  double *Phi1 = nullptr, *Phi2 = nullptr, *Phi3 = nullptr, *D32 = nullptr;
+  // kept for the stages' initial guesses (Instance), and the dt of the last fused RK call (0: none)
+  double *Pl = nullptr, *eend = nullptr, *pend = nullptr;
+  float* H = nullptr;
+  int* hist_d = nullptr;
   // column positions on the host, and the cos/sin(k x) table of the left-zone columns for the
   // generated signal (its own device block, rebuilt by sem_set_wave_input)
   std::vector<double> xcol_h;
   double* wkx = nullptr;
   double hist_dt = 0.0;
-  const double *hist_eta = nullptr, *hist_phis = nullptr;
   unsigned int* stage_bars = nullptr;   // barrier pair of this mesh's own fused stage launch
   int stage_team = 0;
   size_t stage_smem = 0;         // the mesh's own fused stage launch (with the factor cache)
@@ -323,15 +323,6 @@ int do_rhs(sem_mesh* m, const double* eta, const double* phis, double time, doub
   return SEM_OK;
 }
 
-// After a fused RK call: the next call continues the trajectory if it steps the same state
-// buffers with the same dt (then its stages 2 and 3 may extrapolate from the last step's stage
-// potentials).
-void set_history(sem_mesh* m, const double* eta, const double* phis, double dt) {
-  m->hist_dt = dt;
-  m->hist_eta = eta;
-  m->hist_phis = phis;
-}
-
 // own_launch: the mesh's own fused stage launch, whose shared memory holds the factor cache.
 // chunk > 0: element columns per pass in a batch launch.
 Instance make_instance(sem_mesh* m, double* eta, double* phis, double tstart, double dt, int team0,
@@ -349,8 +340,8 @@ Instance make_instance(sem_mesh* m, double* eta, double* phis, double tstart, do
   I.s0e = m->se; I.s0p = m->sp; I.s1e = m->s1e; I.s1p = m->s1p;
   I.ke = m->ke; I.kp = m->kp; I.ae = m->ae; I.ap = m->ap;
   I.wt = m->wt; I.R = m->R; I.R2 = m->R2; I.ub = m->ub; I.ub_stride = m->p.Nx + m->grid + 1;
-  I.P1 = m->Phi1; I.P2 = m->Phi2; I.P3 = m->Phi3; I.D32 = m->D32;
-  I.hist = (m->hist_dt == dt && m->hist_eta == eta && m->hist_phis == phis) ? 1 : 0;
+  I.Pl = m->Pl; I.H = m->H; I.hist_d = m->hist_d; I.eend = m->eend; I.pend = m->pend;
+  I.hist = m->hist_dt == dt ? 1 : 0;
   I.tstart = tstart; I.dt = dt;
   I.tau = m->p.relax_tau > 0.0 ? m->p.relax_tau : dt;
   I.team0 = team0; I.nteam = nteam;
@@ -384,7 +375,7 @@ int do_rk4_fused(sem_mesh* m, double* eta, double* phis, double t0, double dt, i
       const int rc = launch_own_stage(m, a, s);
       if (rc) return rc;
     }
-  if (nsteps > 0) set_history(m, eta, phis, dt);
+  if (nsteps > 0) m->hist_dt = dt;
   return SEM_OK;
 }
 
@@ -717,8 +708,8 @@ static int mesh_create_impl(const sem_params* pin, const double* x_edges_h, cons
                o_ap = cv.take<double>(ncol), o_se = cv.take<double>(ncol), o_sp = cv.take<double>(ncol),
                o_etad = cv.take<double>(ncol), o_phisd = cv.take<double>(ncol),
                o_s1e = cv.take<double>(ncol), o_s1p = cv.take<double>(ncol),
-               o_P1 = cv.take<double>(n), o_P2 = cv.take<double>(n), o_P3 = cv.take<double>(n),
-               o_D32 = cv.take<double>(n);
+               o_Pl = cv.take<double>(n), o_H = cv.take<float>((size_t)4 * kHist * n), o_hist = cv.take<int>(4),
+               o_eend = cv.take<double>(ncol), o_pend = cv.take<double>(ncol);
   const size_t o_gglob = cv.take<double>((size_t)3 * Nx * Nz * Q * Q);
   const size_t o_sbar = cv.take<unsigned>(4);
   const size_t total = cv.off + 256;
@@ -830,7 +821,8 @@ static int mesh_create_impl(const sem_params* pin, const double* x_edges_h, cons
   m->ke = D_(o_ke); m->kp = D_(o_kp); m->ae = D_(o_ae); m->ap = D_(o_ap); m->se = D_(o_se); m->sp = D_(o_sp);
   m->eta_dev = D_(o_etad); m->phis_dev = D_(o_phisd);
   m->s1e = D_(o_s1e); m->s1p = D_(o_s1p);
-  m->Phi1 = D_(o_P1); m->Phi2 = D_(o_P2); m->Phi3 = D_(o_P3); m->D32 = D_(o_D32);
+  m->Pl = D_(o_Pl); m->H = F_(o_H); m->hist_d = reinterpret_cast<int*>(m->pool + o_hist);
+  m->eend = D_(o_eend); m->pend = D_(o_pend);
   m->stage_bars = reinterpret_cast<unsigned int*>(m->pool + o_sbar);
 
   SurfTables& t = m->st;
@@ -1558,7 +1550,7 @@ int sem_batch_rk4_step(sem_batch* b, double* const* eta_d, double* const* phis_d
         }
   }
   if (nsteps > 0)
-    for (int i = 0; i < n; ++i) set_history(b->meshes[i], eta_d[i], phis_d[i], dt_h[i]);
+    for (int i = 0; i < n; ++i) b->meshes[i]->hist_dt = dt_h[i];
   int rc = batch_status(b, plan, s);
   if (t_h)
     for (int i = 0; i < n; ++i) t_h[i] += nsteps * dt_h[i];

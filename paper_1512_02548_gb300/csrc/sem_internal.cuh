@@ -203,13 +203,20 @@ struct Instance {
   double *ke, *kp, *ae, *ap;
   double *wt, *R, *R2, *ub;
   int ub_stride;         // ub[2][ub_stride]: interface unknowns of the M' solves, CTA of rank r at e0 + r
-  double *P1, *P2, *P3;  // stage potentials: P1, P2 of this step, P3 of the last stage 3
-  double *D32;           // Φ₃ − Φ₂ of the last step
+  // initial guesses (stage_body): the last stage's potential, backward differences of the stage
+  // increments H[stage − 1][0..kHist−1][n], how many steps they span and a broken-off mark (hist_d[0], [1]), and
+  // the state at the end of the last step
+  double* Pl;
+  float* H;
+  int* hist_d;
+  double *eend, *pend;
   double tstart, dt, tau;
   int team0, nteam;      // first CTA and number of CTAs of this instance's team
   int relax;
-  int hist;              // P3 belongs to the step before this call's first step (same trajectory)
+  int hist;              // the last call stepped with the same dt (its end state decides on the device)
 };
+
+constexpr int kHist = 4;   // backward differences kept per stage (cubic extrapolation over the steps)
 
 struct StageArgs {
   const Instance* inst;  // device array; nullptr: the one instance `own`
