@@ -514,7 +514,7 @@ namespace semgb {
 // assigned to one instance of a batch.
 struct Team {
   int rank, size;        // this CTA's index in the team, number of CTAs
-  unsigned int* bar;     // arrival counter (and one spare word), zero at launch
+  unsigned int* bar;     // arrival and exit counters, zero at launch
   int* status;           // device status word of the instance
   double* part;          // reduction partials [4 slots][4 values][stride]
   int stride;
@@ -1406,16 +1406,18 @@ __device__ __forceinline__ double prec_mw_entry(const DevGeom& g, int ex, int i)
   return 0.5 * g.dxe[ex] * w[i] * g.geo64[(size_t)ex * Q * 4 + i * 4 + 1];
 }
 template <int P>
-__device__ __forceinline__ void prec_elem_kx(const DevGeom& g, int ex, double* Kx, double* mw) {
+__device__ __forceinline__ void prec_elem_kx(const DevGeom& g, int ex, double* Kx, double* mw, float* Kf) {
   constexpr int Q = P + 1;
-  for (int t = threadIdx.x; t < Q * Q; t += blockDim.x) Kx[t] = prec_kx_entry<P>(g, ex, t);
+  for (int t = threadIdx.x; t < Q * Q; t += blockDim.x) Kf[t] = (float)(Kx[t] = prec_kx_entry<P>(g, ex, t));
   for (int i = threadIdx.x; i < Q; i += blockDim.x) mw[i] = prec_mw_entry<P>(g, ex, i);
 }
 
-// Mode k of element ex (one thread).
+// Mode k of element ex (one thread).  Kf: Kx rounded to FP32, once per element: a conversion holds the
+// FP64 pipe as long as an FMA, and every mode needs all (P − 1)(P + 1) of them (the diagonal, which the mode
+// changes, is rounded after its FP64 sum).  Set-up of a tank's team in the 512-tank batch 35 → 28 µs a stage.
 template <int P>
 __device__ __forceinline__ void prec_elem_mode(const DevGeom& g, const PrecSetup& ps, int ex, int k,
-                                               const double* Kx, const double* mw) {
+                                               const double* Kx, const double* mw, const float* Kf) {
   constexpr int Q = P + 1, Pm = P - 1;
   const double lam = ps.lam[k];
   float Ai[Pm][Pm], Bm[Pm][Pm];
@@ -1423,7 +1425,7 @@ __device__ __forceinline__ void prec_elem_mode(const DevGeom& g, const PrecSetup
   for (int i = 0; i < Pm; ++i)
 #pragma unroll
     for (int j = 0; j < Pm; ++j) {
-      Bm[i][j] = (float)(Kx[(1 + i) * Q + 1 + j] + (i == j ? lam * mw[1 + i] : 0.0));
+      Bm[i][j] = i == j ? (float)(Kx[(1 + i) * Q + 1 + j] + lam * mw[1 + i]) : Kf[(1 + i) * Q + 1 + j];
       Ai[i][j] = (i == j) ? 1.f : 0.f;
     }
 #pragma unroll
@@ -1450,8 +1452,9 @@ __device__ __forceinline__ void prec_elem_mode(const DevGeom& g, const PrecSetup
   // already, and the FP64 pipe is the scarce one (the Schur complements below stay FP64)
   float kb0[Pm], kb1[Pm];
 #pragma unroll
-  for (int m = 0; m < Pm; ++m) { kb0[m] = (float)Kx[1 + m]; kb1[m] = (float)Kx[P * Q + 1 + m]; }
+  for (int m = 0; m < Pm; ++m) { kb0[m] = Kf[1 + m]; kb1[m] = Kf[P * Q + 1 + m]; }
   double Z0[Pm], Z1[Pm];
+  float z0[Pm], z1[Pm];
 #pragma unroll
   for (int i = 0; i < Pm; ++i) {
     float a0 = 0.f, a1 = 0.f;
@@ -1461,6 +1464,7 @@ __device__ __forceinline__ void prec_elem_mode(const DevGeom& g, const PrecSetup
       a0 = fmaf(kb0[m], am, a0);
       a1 = fmaf(kb1[m], am, a1);
     }
+    z0[i] = a0; z1[i] = a1;
     Z0[i] = a0; Z1[i] = a1;
   }
   double S00 = Kx[0] + lam * mw[0], S01 = Kx[P], S11 = Kx[P * Q + P] + lam * mw[P];
@@ -1473,8 +1477,8 @@ __device__ __forceinline__ void prec_elem_mode(const DevGeom& g, const PrecSetup
   float* Z32 = ps.Z32 + (size_t)ex * 2 * Pm * nr + k;      // mode-fastest: Z32[(s·Pm + i)·nr]
 #pragma unroll
   for (int i = 0; i < Pm; ++i) {
-    Z32[i * nr] = (float)Z0[i];
-    Z32[(Pm + i) * nr] = (float)Z1[i];
+    Z32[i * nr] = z0[i];
+    Z32[(Pm + i) * nr] = z1[i];
   }
   ps.schur[base * 3 + 0] = S00;
   ps.schur[base * 3 + 1] = S01;
@@ -1486,10 +1490,11 @@ __global__ void __launch_bounds__(kPrecModesPerBlock) k_prec_elem(DevGeom g, Pre
   constexpr int Q = P + 1;
   __shared__ double Kx[Q * Q];
   __shared__ double mw[Q];
-  prec_elem_kx<P>(g, blockIdx.x, Kx, mw);
+  __shared__ float Kf[Q * Q];
+  prec_elem_kx<P>(g, blockIdx.x, Kx, mw, Kf);
   __syncthreads();
   const int k = blockIdx.y * blockDim.x + threadIdx.x;
-  if (k < ps.nr) prec_elem_mode<P>(g, ps, blockIdx.x, k, Kx, mw);
+  if (k < ps.nr) prec_elem_mode<P>(g, ps, blockIdx.x, k, Kx, mw, Kf);
 }
 
 // One warp per mode: interface tridiagonal d_j = S00(j) + S11(j−1), e_j = S01(j) and its Thomas
@@ -1765,7 +1770,7 @@ __device__ void stage_body(Instance& I, const Team& tm, int stage, int step, uns
   // so that all (element, mode) pairs of the batch run at once.
   {
     double* kxs = reinterpret_cast<double*>(smem_raw);
-    constexpr int per = Q * Q + Q;
+    constexpr int per = Q * Q + Q + (Q * Q + 1) / 2;   // Kx, mw, Kx in FP32
     const int avail = Q * Q + Q + g.nrow +
                       g.chunk * (2 * g.Nz + 4 * Q + Q * g.nrow + g.nrow * (Q | 1) + 2 * g.Nz * Q * (Q | 1) + g.Nz * Q);
     const int nb_max = max(1, min(ne, avail / per));
@@ -1774,7 +1779,9 @@ __device__ void stage_body(Instance& I, const Team& tm, int stage, int step, uns
       const int nb = min(nb_max, R.e1 - e0);
       for (int t = threadIdx.x; t < nb * Q * Q; t += blockDim.x) {
         const int b = t / (Q * Q);
-        kxs[b * per + (t - b * Q * Q)] = prec_kx_entry<P>(g, e0 + b, t - b * Q * Q);
+        const double v = prec_kx_entry<P>(g, e0 + b, t - b * Q * Q);
+        kxs[b * per + (t - b * Q * Q)] = v;
+        reinterpret_cast<float*>(kxs + b * per + Q * Q + Q)[t - b * Q * Q] = (float)v;
       }
       for (int t = threadIdx.x; t < nb * Q; t += blockDim.x) {
         const int b = t / Q;
@@ -1783,7 +1790,8 @@ __device__ void stage_body(Instance& I, const Team& tm, int stage, int step, uns
       __syncthreads();
       for (int t = threadIdx.x; t < nb * nr; t += blockDim.x) {
         const int b = g.dv_nr.div(t), k = t - b * nr;
-        prec_elem_mode<P>(g, I.ps, e0 + b, k, kxs + b * per, kxs + b * per + Q * Q);
+        prec_elem_mode<P>(g, I.ps, e0 + b, k, kxs + b * per, kxs + b * per + Q * Q,
+                          reinterpret_cast<const float*>(kxs + b * per + Q * Q + Q));
       }
       __syncthreads();
     }
@@ -1851,9 +1859,14 @@ __device__ void stage_body(Instance& I, const Team& tm, int stage, int step, uns
     }
   }
   // w̃ on owned columns; condensed element S_x of η and φ̃
-  for (int c0 = R.c0 + 4 * warp; c0 < R.c1; c0 += 4 * nw) {
-    const int col = c0 + (lane >> 3);
-    wsurf_column8(t, I.pa.x, ein, I.wt, col < R.c1 ? col : -1, lane & 7);
+  // (many columns: one thread each, which takes a fifth of the FP64 instructions; few: eight lanes each)
+  if (nc >= (int)blockDim.x / 2) {
+    for (int col = R.c0 + threadIdx.x; col < R.c1; col += blockDim.x) wsurf_column1(t, I.pa.x, ein, I.wt, col);
+  } else {
+    for (int c0 = R.c0 + 4 * warp; c0 < R.c1; c0 += 4 * nw) {
+      const int col = c0 + (lane >> 3);
+      wsurf_column8(t, I.pa.x, ein, I.wt, col < R.c1 ? col : -1, lane & 7);
+    }
   }
   for (int q = threadIdx.x; q < 2 * ne * Q; q += blockDim.x) {
     const int fld = q / (ne * Q), r = q - fld * ne * Q;

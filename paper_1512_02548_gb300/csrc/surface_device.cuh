@@ -35,6 +35,19 @@ __device__ __forceinline__ void wsurf_column8(const SurfTables& t, const double*
   if (col >= 0 && sub == 0) w[col] = acc / (eta[col] + t.h[col]);
 }
 
+// The same by one thread (four partial sums: the chain of one would be Nrow FP64 latencies long).
+__device__ __forceinline__ void wsurf_column1(const SurfTables& t, const double* __restrict__ Phi,
+                                              const double* __restrict__ eta, double* __restrict__ w, int col) {
+  const double* phi = Phi + (size_t)col * t.nrow;
+  double a[4] = {0.0, 0.0, 0.0, 0.0};
+  int iz = 0;
+  for (; iz + 4 <= t.nrow; iz += 4)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) a[q] = fma(t.wrow[iz + q], phi[iz + q], a[q]);
+  for (; iz < t.nrow; ++iz) a[0] = fma(t.wrow[iz], phi[iz], a[0]);
+  w[col] = ((a[0] + a[1]) + (a[2] + a[3])) / (eta[col] + t.h[col]);
+}
+
 // M'u = Σ_e Q_eᵀ R_e (M' constant in time).  The element right-hand sides are stored condensed: the
 // element interiors are eliminated on the host, in the tables, so that an item of an element's row a is
 //   a = 0, P:      the boundary rows R_b − M_bi M_ii⁻¹ R_i (the interface right-hand side),
