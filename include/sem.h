@@ -304,7 +304,8 @@ int sem_batch_rk4_step_host(sem_batch* b, double* eta_h, double* phis_h, double*
 typedef struct sem_batch_tuning {
   double cluster_share;  /* cluster plan: a team is the smallest power of two of CTAs whose work per
                             CTA is at most this fraction of the batch's work per CTA slot (0.5)   */
-  int max_cluster;       /* largest cluster team, a power of two in 1..16 (16)                   */
+  int max_cluster;       /* largest cluster team, a power of two in 1..16 (16); the plan takes teams of
+                            at most 4, 8 or 16 of these, by its estimate                         */
   int narrow_max;        /* groups of at most this many instances use the one-CTA-per-SM build (8) */
   int plan;              /* -1: the plan estimated faster; 0: cooperative; 1: clusters (-1)       */
 } sem_batch_tuning;

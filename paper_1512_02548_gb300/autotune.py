@@ -110,7 +110,7 @@ def tune_batch(dev, count: int = 512, seed: int = 1, steps: int = 3, quick: bool
     wls = c3_instances(count, seed=seed)
     init = [initial_state(wl, _column_x(wl), np.full(wl.ncol, wl.depth)) for wl in wls]
     shares = (0.25, 0.5, 1.0) if quick else (0.125, 0.25, 0.5, 1.0, 2.0)
-    clusters = (8, 16) if quick else (4, 8, 16)
+    clusters = (16,)   # the planner takes clusters of at most 4, 8 or 16 by its estimate
     narrows = (8,) if quick else (8, 1 << 20)
     rows = []
     for share, mc, nm in itertools.product(shares, clusters, narrows):

@@ -1205,30 +1205,39 @@ int plan_cooperative(sem_batch* b, sem_mesh* const* meshes, int count, int sms) 
   return SEM_OK;
 }
 
-// Cluster plan: each member's team is one thread-block cluster, so no CTA waits on a CTA outside
-// its cluster; the launches need no co-residency, the hardware starts clusters as CTA slots free
-// up, and the launches of all groups run at the same time on streams of their own.  A step then
-// lasts about the larger of the total work per CTA slot and the longest team's time, so a member's
-// team is the smallest power of two c ≤ 16 (and ≤ its buffer limit) whose work per CTA is at most
-// half the total work per CTA slot (work: element-local nodes × the apply's flops per node).
-// Members are grouped by (order, precision, c), the largest first within a launch.  Returns
-// false (and builds nothing) when some group's cluster does not fit on the device.
 double member_work(const sem_mesh* m) {
   const int Q = m->p.P + 1;
   return (double)m->p.Nx * m->p.Nz * Q * Q * (8.0 * Q + 7.0);
 }
 
-// Estimated step time of each plan, in units of work per CTA: the cluster plan's launches share the
-// GPU, so it takes about the larger of the total work per CTA slot and its longest team; the
-// cooperative plan's launches run one after another, each as long as its slowest team.
-double estimate_clusters(const sem_batch* b, double slots) {
+// Estimated stage times of the plans, in units of work (element-local nodes × the apply's flops per node:
+// about 2 ns of a CTA).  A CTA's stage costs its share of its tank's work plus its chain of phases and
+// barriers, kChainWork (130 µs).  Cluster launches share the GPU: the larger of the sum of that over the CTA
+// slots and of the longest team's.  Cooperative launches run one after another, each as long as its slowest
+// team plus kCoopWork (80 µs: fewer, larger teams a launch, but launched once per order).  Measured RK4 steps
+// of uneven tanks of five orders, ms, with cluster caps of 4 / 8 / 16 and cooperative: 8 tanks – / – / 0.75 / 2.03;
+// 30: – / – / 1.65 / 2.39; 100: – / – / 3.84 / 3.24; 200: – / 4.70 / 5.65 / 4.79; 512: 9.67 / 10.27 / 10.85 /
+// 10.97 (share 0.25; with the re-measured share of 0.5 the plan takes 0.75, 1.65, 2.66, 4.54 and 9.42).  24 Laplace
+// solves of 1e3 to 2e5 nodes, cap 16 against cooperative: 6.69 / 5.59.
+constexpr double kChainWork = 6.5e4, kCoopWork = 4.0e4;
+
+// Cluster size of a member: the smallest power of two (≤ cap and its buffer limit) whose work per CTA is at
+// most the tuned share of the batch's work per CTA slot.
+int cluster_size(const sem_mesh* m, double w, double per_cta, int cap) {
+  const int cmax = std::min(cap, batch_limit(m));
+  const double want = per_cta > 0.0 ? w / per_cta : 1.0;
+  int c = 1;
+  while (c < want && 2 * c <= cmax) c *= 2;
+  return c;
+}
+
+double estimate_clusters(sem_mesh* const* meshes, const std::vector<double>& w, double per_cta, int cap, double slots) {
   double total = 0.0, longest = 0.0;
-  for (const auto& L : b->cl_launches)
-    for (size_t k = 0; k < L.members.size(); ++k) {
-      const double w = member_work(b->meshes[L.members[k]]);
-      total += w;
-      longest = std::max(longest, w / L.nteam[k]);
-    }
+  for (size_t i = 0; i < w.size(); ++i) {
+    const int c = cluster_size(meshes[i], w[i], per_cta, cap);
+    total += w[i] + c * kChainWork;
+    longest = std::max(longest, w[i] / c + kChainWork);
+  }
   return std::max(total / slots, longest);
 }
 
@@ -1238,12 +1247,19 @@ double estimate_cooperative(const sem_batch* b) {
     double worst = 0.0;
     for (size_t k = 0; k < L.members.size(); ++k)
       worst = std::max(worst, member_work(b->meshes[L.members[k]]) / L.nteam[k]);
-    t += worst;
+    t += worst + kCoopWork;
   }
   return t;
 }
 
-bool plan_clusters(sem_batch* b, sem_mesh* const* meshes, int count, int sms) {
+// Cluster plan: each member's team is one thread-block cluster, so no CTA waits on a CTA outside
+// its cluster; the launches need no co-residency, the hardware starts clusters as CTA slots free
+// up, and the launches of all groups run at the same time on streams of their own.  The largest
+// cluster is the one of 4, 8 and 16 CTAs (at most the tuned maximum) with the best estimate: few tanks
+// are bound by the longest team, many by the CTA slots, where every further CTA costs its chain.
+// Members are grouped by (order, precision, c), the largest first within a launch.  Returns
+// false (and builds nothing) when some group's cluster does not fit on the device; *estimate: its stage time.
+bool plan_clusters(sem_batch* b, sem_mesh* const* meshes, int count, int sms, double* estimate) {
   std::vector<double> w(count);
   double total = 0.0;
   for (int i = 0; i < count; ++i) {
@@ -1253,12 +1269,15 @@ bool plan_clusters(sem_batch* b, sem_mesh* const* meshes, int count, int sms) {
   const sem_batch_tuning tune = batch_tuning();
   const double slots = 2.0 * sms;
   const double per_cta = tune.cluster_share * total / slots;
+  int cap = std::min(4, tune.max_cluster);
+  *estimate = estimate_clusters(meshes, w, per_cta, cap, slots);
+  for (int c = 8; c <= tune.max_cluster; c *= 2) {
+    const double e = estimate_clusters(meshes, w, per_cta, c, slots);
+    if (e < *estimate) { *estimate = e; cap = c; }
+  }
   std::vector<std::pair<std::array<int, 3>, std::vector<int>>> groups;
   for (int i = 0; i < count; ++i) {
-    const int cmax = std::min(tune.max_cluster, batch_limit(meshes[i]));
-    const double want = per_cta > 0.0 ? w[i] / per_cta : 1.0;
-    int c = 1;
-    while (c < want && 2 * c <= cmax) c *= 2;
+    const int c = cluster_size(meshes[i], w[i], per_cta, cap);
     const std::array<int, 3> key{meshes[i]->p.P, meshes[i]->p.precision == SEM_PREC_MIXED ? 1 : 0, c};
     auto it = std::find_if(groups.begin(), groups.end(), [&](const auto& g) { return g.first == key; });
     if (it == groups.end()) groups.push_back({key, {i}});
@@ -1391,8 +1410,8 @@ int sem_batch_create(sem_mesh* const* meshes, int count, sem_batch** out) {
   // forces either plan.
   const char* cenv = std::getenv("SEM_BATCH_CLUSTER");
   const int force = cenv ? (std::atoi(cenv) != 0 ? 1 : 0) : batch_tuning().plan;
-  if (force != 0 && plan_clusters(b, meshes, count, sms) && force < 0 &&
-      estimate_clusters(b, 2.0 * sms) > estimate_cooperative(b))
+  double est = 0.0;
+  if (force != 0 && plan_clusters(b, meshes, count, sms, &est) && force < 0 && est > estimate_cooperative(b))
     b->cl_launches.clear();
   for (int i = 0; i < count; ++i) {
     b->off.push_back(b->ncol_total);
