@@ -707,11 +707,14 @@ static int mesh_create_impl(const sem_params* pin, const double* x_edges_h, cons
                o_ke = cv.take<double>(ncol), o_kp = cv.take<double>(ncol), o_ae = cv.take<double>(ncol),
                o_ap = cv.take<double>(ncol), o_se = cv.take<double>(ncol), o_sp = cv.take<double>(ncol),
                o_etad = cv.take<double>(ncol), o_phisd = cv.take<double>(ncol),
-               o_s1e = cv.take<double>(ncol), o_s1p = cv.take<double>(ncol),
-               o_Pl = cv.take<double>(n), o_H = cv.take<float>((size_t)4 * kHist * n), o_hist = cv.take<int>(4),
-               o_eend = cv.take<double>(ncol), o_pend = cv.take<double>(ncol);
-  const size_t o_gglob = cv.take<double>((size_t)3 * Nx * Nz * Q * Q);
+               o_s1e = cv.take<double>(ncol), o_s1p = cv.take<double>(ncol);
+  const size_t o_hist = cv.take<int>(4);
   const size_t o_sbar = cv.take<unsigned>(4);
+  // written before they are read (the factor cache by every solve, the guess history by the first step of a
+  // trajectory, which hist_d[0] = 0 marks): not cleared
+  const size_t clear_end = cv.off;
+  const size_t o_gglob = cv.take<double>((size_t)3 * Nx * Nz * Q * Q), o_Pl = cv.take<double>(n),
+               o_H = cv.take<float>((size_t)4 * kHist * n), o_eend = cv.take<double>(ncol), o_pend = cv.take<double>(ncol);
   const size_t total = cv.off + 256;
   if (footprint_only) {
     *footprint_only = total;
@@ -731,7 +734,7 @@ static int mesh_create_impl(const sem_params* pin, const double* x_edges_h, cons
     if (!v.empty()) std::memcpy(stage.data() + o, v.data(), v.size() * sizeof(double));
   };
   {
-    cudaError_t e = cudaMemset(m->pool + up_end, 0, total - up_end);
+    cudaError_t e = cudaMemset(m->pool + up_end, 0, clear_end - up_end);
     if (e != cudaSuccess) code = fail(SEM_ERR_CUDA, std::string("memset: ") + cudaGetErrorString(e));
   }
   up(o_h, std::vector<double>(h_h, h_h + ncol));
