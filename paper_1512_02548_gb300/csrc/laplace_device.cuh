@@ -2166,7 +2166,7 @@ constexpr int kElemMaxP = 8;
 template <int P>
 static bool elem_fills(const DevGeom& g) {
   const int E = g.Nz == 1 ? ElemTile<P, 1>::E : g.Nz == 2 ? ElemTile<P, 2>::E : g.Nz == 3 ? ElemTile<P, 3>::E : ElemTile<P, 4>::E;
-  return g.Nx >= 152 * E;
+  return g.Nx >= (P <= 6 ? 76 : 152) * E;
 }
 
 template <int P, int NZ>
@@ -2211,8 +2211,9 @@ cudaError_t launch_apply_tile_impl(int fp32, const DevGeom& g, const void* x, vo
   }
   if constexpr (P <= kElemMaxP) {
     // one element per thread; orders 7 and 8 (255 registers, 2 CTAs an SM) from the size on that gives
-    // every SM a tile: 2.5 M nodes at P = 8 take 23–27 → 17–23 µs, 0.6 M nodes 10–12 → 14–16
-    if (fp32 && g.Nz <= 4 && (P <= 6 || elem_fills<P>(g))) {
+    // every SM a tile: 2.5 M nodes at P = 8 take 23–27 → 17–23 µs, 0.6 M nodes 10–12 → 14–16; order 6 with one
+    // layer (tiles of 127 elements) from half of that: 0.6 M nodes 12.3 → 10.3 µs, 0.16 M 9.3 → 10.2
+    if (fp32 && g.Nz <= 4 && (P <= 5 || (P == 6 && g.Nz > 1) || elem_fills<P>(g))) {
       const int vec_ok = (reinterpret_cast<uintptr_t>(y) % 16) == 0 ? 1 : 0;
       switch (g.Nz) {
         case 1: return launch_apply_elem<P, 1>(g, xf, yf, bulk_ok, vec_ok, s);

@@ -67,3 +67,20 @@ def test_many_tiles_per_cta_match_the_fp64_apply():
     m.laplace_apply_f32(x, y)
     m.laplace_apply(x.double(), y64)
     assert float(torch.linalg.norm(y.double() - y64) / torch.linalg.norm(y64)) < 2e-6
+
+
+@pytest.mark.parametrize("P,Nz", [(6, 1), (7, 1), (7, 2), (7, 3), (7, 4), (8, 1), (8, 2), (8, 3), (8, 4)])
+@pytest.mark.parametrize("periodic", [True, False])
+def test_orders_that_take_it_from_a_size_on(P, Nz, periodic):
+    # the first size of the rule and one element more (a ragged last tile), against the FP64 apply
+    for Nx in (152 * TILE[Nz], 152 * TILE[Nz] + 1):
+        wl = small_case(P=P, Nx=Nx, Nz=Nz, periodic=periodic)
+        wl.length = 2 * np.pi * Nx / 64
+        m = sem.Mesh.from_workload(wl, h=np.ones(wl.ncol))
+        x = torch.randn(m.n, dtype=torch.float32, device=DEV)
+        m.update_geometry(0.01 * torch.sin(torch.arange(m.ncol, dtype=torch.float64, device=DEV) * 0.01))
+        y, y64 = torch.empty_like(x), torch.empty(m.n, dtype=torch.float64, device=DEV)
+        m.laplace_apply_f32(x, y)
+        m.laplace_apply(x.double(), y64)
+        assert float(torch.linalg.norm(y.double() - y64) / torch.linalg.norm(y64)) < 2e-6
+        m.close()
