@@ -210,7 +210,9 @@ int sem_laplace_solve(sem_mesh* m, const double* phis_d, double* Phi_d,
  * (eq. velocpot2), and the C⁰ derivatives from M'u = S_x f (eq.
  * representationU) for f = η and f = φ̃.  Uses the geometry of the last
  * sem_update_geometry (for 1/d).  Inputs Phi_d (n), eta_d, phis_d (Ncol);
- * outputs w_surf_d, etax_d, phisx_d (Ncol each); all device. */
+ * outputs w_surf_d, etax_d, phisx_d (Ncol each); all device.  An output may lie over an
+ * input (etax_d = eta_d, say): the inputs count as they were before the call, and
+ * outputs over one another are written in the order of the arguments.  That costs three copies. */
 int sem_recover_gradient(sem_mesh* m, const double* Phi_d, const double* eta_d,
                          const double* phis_d, double* w_surf_d, double* etax_d,
                          double* phisx_d, void* stream);

@@ -5,6 +5,7 @@
 #include <array>
 #include <atomic>
 #include <cmath>
+#include <cstdint>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -294,6 +295,12 @@ int do_geometry(sem_mesh* m, const double* eta, cudaStream_t s) {
   CUDA_TRY(launch_geometry(m->g, eta, jacobi, s));
   if (!jacobi) CUDA_TRY(launch_prec_setup(m->g, m->ps, s));
   return SEM_OK;
+}
+
+// Do na doubles at a and nb doubles at b share an address?
+bool overlap(const double* a, size_t na, const double* b, size_t nb) {
+  const uintptr_t pa = reinterpret_cast<uintptr_t>(a), pb = reinterpret_cast<uintptr_t>(b);
+  return pa < pb + nb * sizeof(double) && pb < pa + na * sizeof(double);
 }
 
 bool has_zones(const sem_mesh* m) { return m->p.relax_left > 0.0 || m->p.relax_right > 0.0; }
@@ -978,7 +985,24 @@ int sem_recover_gradient(sem_mesh* m, const double* Phi_d, const double* eta_d, 
     return fail(SEM_ERR_INVALID_ARG, "NULL argument");
   DeviceGuard dg(m->device);
   cudaStream_t s = (cudaStream_t)stream;
-  CUDA_TRY(launch_recover(m->st, Phi_d, eta_d, phis_d, w_surf_d, etax_d, phisx_d, s));
+  // The kernel's blocks store while others still read the state around their own elements: where an output
+  // lies over an input or another output, the results are complete before they are copied there.
+  const double* in[3] = {Phi_d, eta_d, phis_d};
+  const size_t n_in[3] = {(size_t)m->n, (size_t)m->ncol, (size_t)m->ncol}, nc = (size_t)m->ncol;
+  double* out[3] = {w_surf_d, etax_d, phisx_d};
+  double* tmp[3] = {m->wt, m->etax, m->phisx};
+  bool shared = false;
+  for (int i = 0; i < 3; ++i) {
+    for (int j = 0; j < 3; ++j) shared = shared || overlap(out[i], nc, in[j], n_in[j]);
+    for (int j = 0; j < i; ++j) shared = shared || overlap(out[i], nc, out[j], nc);
+  }
+  if (!shared) {
+    CUDA_TRY(launch_recover(m->st, Phi_d, eta_d, phis_d, w_surf_d, etax_d, phisx_d, s));
+    return SEM_OK;
+  }
+  CUDA_TRY(launch_recover(m->st, Phi_d, eta_d, phis_d, tmp[0], tmp[1], tmp[2], s));
+  for (int i = 0; i < 3; ++i)
+    CUDA_TRY(cudaMemcpyAsync(out[i], tmp[i], nc * sizeof(double), cudaMemcpyDeviceToDevice, s));
   return SEM_OK;
 }
 
