@@ -250,7 +250,9 @@ int sem_apply_filter(sem_mesh* m, double* q_d, void* stream);
  * Ncol.  Synchronises once at the end.  Each stage's Laplace solve starts from an
  * extrapolation of earlier stage potentials kept by the mesh, over up to four steps of the
  * trajectory.  A call continues the last call's trajectory when its state equals, value by value, the
- * state that the last step of this mesh left, and dt is the same; any other state starts anew.
+ * state that the last step of this mesh left, and dt is the same.  After a small change of that state by the
+ * caller (a filter, forcing or absorption of its own; up to 1/16 of the largest eta and phis) stages 2 to 4 still
+ * start from their extrapolations and stage 1 from the last potential; any other state starts anew.
  * The starting point does not change the converged result, only the iteration count; a failed step
  * clears the history. */
 int sem_rk4_step(sem_mesh* m, double* eta_d, double* phis_d, double* t, double dt,

@@ -164,7 +164,7 @@ struct sem_mesh {
   double *ke = nullptr, *kp = nullptr, *ae = nullptr, *ap = nullptr, *se = nullptr, *sp = nullptr;
   double *eta_dev = nullptr, *phis_dev = nullptr;
   double *s1e = nullptr, *s1p = nullptr;   // second stage-input pair of the fused RK stage
-  // kept for the stages' initial guesses (Instance), and the dt of the last fused RK call (0: none)
+  // kept for the stages' initial guesses (Instance), and the dt of the last fused RK call (NaN: none)
   double *Pl = nullptr, *eend = nullptr, *pend = nullptr;
   float* H = nullptr;
   int* hist_d = nullptr;
@@ -172,7 +172,7 @@ struct sem_mesh {
   // generated signal (its own device block, rebuilt by sem_set_wave_input)
   std::vector<double> xcol_h;
   double* wkx = nullptr;
-  double hist_dt = 0.0;
+  double hist_dt = NAN;
   unsigned int* stage_bars = nullptr;   // barrier pair of this mesh's own fused stage launch
   int stage_team = 0;
   size_t stage_smem = 0;         // the mesh's own fused stage launch (with the factor cache)
@@ -248,7 +248,7 @@ int status_error(int st) {
 // After a failed step the mesh's warm-start potential may hold non-finite values; the next
 // solve on this mesh starts from zero instead.
 cudaError_t reset_warm_start(sem_mesh* m, cudaStream_t s) {
-  m->hist_dt = 0.0;   // the stage potentials kept for initial guesses may be from a failed step
+  m->hist_dt = NAN;   // the stage potentials kept for initial guesses may be from a failed step
   return cudaMemsetAsync(m->Phi, 0, sizeof(double) * (size_t)m->n, s);
 }
 
@@ -715,7 +715,7 @@ static int mesh_create_impl(const sem_params* pin, const double* x_edges_h, cons
                o_ap = cv.take<double>(ncol), o_se = cv.take<double>(ncol), o_sp = cv.take<double>(ncol),
                o_etad = cv.take<double>(ncol), o_phisd = cv.take<double>(ncol),
                o_s1e = cv.take<double>(ncol), o_s1p = cv.take<double>(ncol);
-  const size_t o_hist = cv.take<int>(4);
+  const size_t o_hist = cv.take<int>(8);
   const size_t o_sbar = cv.take<unsigned>(4);
   // written before they are read (the factor cache by every solve, the guess history by the first step of a
   // trajectory, which hist_d[0] = 0 marks): not cleared

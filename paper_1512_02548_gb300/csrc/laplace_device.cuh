@@ -1748,23 +1748,43 @@ __device__ void stage_body(Instance& I, const Team& tm, int stage, int step, uns
   // differences in FP32 (they steer the start of the solve only).  Relative errors of the guesses of
   // stages 1..4 on a tank of 30×2, P = 6, H/L = 0.02, dt = T/200: 1.5e-10, 2e-8, 6e-10, 2e-8, where extrapolation
   // from the last two or three stage potentials had 2.5e-6, 2.3e-4, 7e-6, 8e-6.
-  // A trajectory continues when this call's state equals, value by value, the state at the end of the
-  // last step and dt is the same; any other state starts a new history (all CTAs agree after the barrier).
+  // A trajectory continues when dt is the same and this call's state equals, value by value, the state at
+  // the end of the last step.  A state that differs a little (the caller's own filter, forcing or absorption
+  // between calls) keeps the increments inside a step, stages 2..4, and starts D_1, which spans the change, and
+  // stage 1, which keeps the last potential, anew.  "A little": at most kTouch of the largest value, of η
+  // and of φ̃.  A cubic extrapolation passes on at most 15 times a relative change of the increments, so below
+  // 1/16 it is still nearer than no extrapolation.  Any other state starts a new history.  The largest
+  // differences and values go through hist_d[2..5] (float bits, rounded up), so all CTAs agree after the barrier.
   const bool keep = stage >= 1 && stage <= 4;
   const size_t nn = (size_t)g.ncol * g.nrow;
   float* Hs = keep ? I.H + (size_t)(stage - 1) * kHist * nn : nullptr;
   const bool entry = stage == 1 && step == 0;
-  if (entry) {
-    bool other = I.hist == 0;
-    for (int col = R.c0 + threadIdx.x; col < R.c1; col += blockDim.x)
-      other = other || I.eta[col] != I.eend[col] || I.phis[col] != I.pend[col];
-    if (other) atomicOr(I.hist_d + 1, 1);
+  const bool compare = entry && I.hist != 0;
+  unsigned* smx = reinterpret_cast<unsigned*>(red);
+  if (compare) {
+    if (threadIdx.x < 4) smx[threadIdx.x] = 0u;
+    __syncthreads();
+    unsigned v[4] = {0u, 0u, 0u, 0u};
+    auto up = [](unsigned& m, double x) { m = max(m, __float_as_uint(__double2float_ru(fabs(x)))); };
+    for (int col = R.c0 + threadIdx.x; col < R.c1; col += blockDim.x) {
+      const double e = I.eend[col], p = I.pend[col];
+      up(v[0], I.eta[col] - e);
+      up(v[1], e);
+      up(v[2], I.phis[col] - p);
+      up(v[3], p);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      v[k] = __reduce_max_sync(0xffffffffu, v[k]);
+      if (lane == 0) atomicMax(smx + k, v[k]);
+    }
   }
   // generated signal of the left relaxation zone at this stage's time: component angles now
   // (all CTAs of the team), the zone columns after the next barrier, read by the relaxation term
   const bool wave_tab = I.relax && t.wkx != nullptr && t.ncomp > 0 && t.nzl > 0 && stage >= 1;
   if (wave_tab) wave_angles(t, time, tm.rank * blockDim.x + threadIdx.x, tm.size * blockDim.x);
   __syncthreads();
+  if (compare && threadIdx.x < 4) atomicMax(reinterpret_cast<unsigned*>(I.hist_d) + 2 + threadIdx.x, smx[threadIdx.x]);
   // preconditioner: condensation of the owned elements for every mode, then interface pivots.
   // The apply's shared memory is free until the solve: it holds Kx and mw of a batch of elements,
   // so that all (element, mode) pairs of the batch run at once.
@@ -1800,12 +1820,20 @@ __device__ void stage_body(Instance& I, const Team& tm, int stage, int step, uns
   if (!grid_barrier(tm, s_flag)) return;
   SEM_MARK(g, tm, TR_BAR_SETUP);
   // the guess, owned nodes only: the next barrier orders these writes before any neighbour reads them
-  int hm = 0;                                  // steps of this trajectory before this one, at most kHist
+  int hm = 0, h1 = 0;                          // steps before this one, at most kHist, kept for stages 2..4 and for stage 1
   if (keep) {
-    hm = entry && __ldcg(I.hist_d + 1) != 0 ? 0 : __ldcg(I.hist_d);
+    if (!entry) {
+      hm = __ldcg(I.hist_d);
+      h1 = __ldcg(I.hist_d + 1);
+    } else if (compare) {
+      auto word = [&](int k) { return __uint_as_float((unsigned)__ldcg(I.hist_d + 2 + k)); };
+      const float de = word(0), dp = word(2);
+      if (de <= kTouch * word(1) && dp <= kTouch * word(3)) hm = __ldcg(I.hist_d);   // not with a NaN
+      if (de == 0.f && dp == 0.f) h1 = __ldcg(I.hist_d + 1);
+    }
     double* x = I.pa.x;
     const int i0 = R.c0 * g.nrow, i1 = R.c1 * g.nrow;
-    if (hm > 0) {
+    if ((stage == 1 ? h1 : hm) > 0) {
       for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
         float v = Hs[i];
 #pragma unroll
@@ -1832,10 +1860,8 @@ __device__ void stage_body(Instance& I, const Team& tm, int stage, int step, uns
   }
   if (!grid_barrier(tm, s_flag)) return;
   SEM_MARK(g, tm, TR_PIVOTS);
-  if (entry && tm.rank == 0 && threadIdx.x == 0) {   // every CTA has read both words
-    if (hm == 0) I.hist_d[0] = 0;
-    I.hist_d[1] = 0;
-  }
+  if (entry && tm.rank == 0 && threadIdx.x < 6)   // every CTA has read them
+    I.hist_d[threadIdx.x] = threadIdx.x == 0 ? hm : threadIdx.x == 1 ? h1 : 0;
   // Laplace solve from the guess
   if (threadIdx.x == 0) I.pa.phis = pin;
   __syncthreads();
@@ -1845,7 +1871,7 @@ __device__ void stage_body(Instance& I, const Team& tm, int stage, int step, uns
   // the stage's increment and its backward differences, for the guesses of the next steps (stage 1: from
   // the trajectory's second step on)
   if (keep) {
-    const int spans = stage == 1 ? hm - 1 : hm;   // earlier increments of this stage
+    const int spans = stage == 1 ? h1 - 1 : hm;   // earlier increments of this stage
     for (int i = R.c0 * g.nrow + threadIdx.x; i < R.c1 * g.nrow; i += blockDim.x) {
       const double v = I.pa.x[i];
       float dn = spans >= 0 ? (float)(v - I.Pl[i]) : 0.f;
@@ -1932,7 +1958,7 @@ __device__ void stage_body(Instance& I, const Team& tm, int stage, int step, uns
       I.eend[col] = I.eta[col];
       I.pend[col] = I.phis[col];
     }
-    if (tm.rank == 0 && threadIdx.x == 0) I.hist_d[0] = min(hm + 1, kHist);
+    if (tm.rank == 0 && threadIdx.x < 2) I.hist_d[threadIdx.x] = min((threadIdx.x ? h1 : hm) + 1, kHist);
   }
 }
 

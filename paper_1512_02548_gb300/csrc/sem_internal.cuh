@@ -204,8 +204,9 @@ struct Instance {
   double *wt, *R, *R2, *ub;
   int ub_stride;         // ub[2][ub_stride]: interface unknowns of the M' solves, CTA of rank r at e0 + r
   // initial guesses (stage_body): the last stage's potential, backward differences of the stage
-  // increments H[stage − 1][0..kHist−1][n], how many steps they span and a broken-off mark (hist_d[0], [1]), and
-  // the state at the end of the last step
+  // increments H[stage − 1][0..kHist−1][n], how many steps they span (hist_d[0]: stages 2..4, [1]: stage 1),
+  // the comparison of a call's state with the last one (hist_d[2..5], zero between launches), and the state
+  // at the end of the last step
   double* Pl;
   float* H;
   int* hist_d;
@@ -217,6 +218,7 @@ struct Instance {
 };
 
 constexpr int kHist = 4;   // backward differences kept per stage (cubic extrapolation over the steps)
+constexpr float kTouch = 1.f / 16;   // a state this near the last end state keeps the increments of stages 2..4
 
 struct StageArgs {
   const Instance* inst;  // device array; nullptr: the one instance `own`
