@@ -20,18 +20,25 @@ namespace semgb {
 // The M' solves run per block of kRecElems elements: the block's window of condensed right-hand sides
 // (its own elements and t.win + 1 more on either side) is enough for its interface unknowns
 // (mass1d_window), so no block waits for another.
-constexpr int kRecElems = 16, kRecThreads = 128;
+constexpr int kRecElems = 16, kRecThreads = 128, kRecCols = kRecThreads / 8;
+__host__ __device__ static inline int rec_blocks(int Nx) { return (Nx + kRecElems - 1) / kRecElems; }
 
-// Gradient recovery: w̃ of the block's columns, S_x of η and φ̃ (boundary rows for the whole window, kept in
-// shared memory), the interface solves and the block's columns of ∂xη and ∂xφ̃.  Latency bound: one
-// launch of Nx/16 blocks instead of three launches, the last of which solved the whole chain on one
-// SM.  1001×2, P = 6, with two filter calls and their copies: 148 → 51 µs, now the host's calls.
+// Gradient recovery, latency bound, in one launch of two kinds of blocks.  The first nrec = Nx/16 take S_x of η
+// and φ̃ (boundary rows for the whole window, kept in shared memory), the interface solves and their
+// columns of ∂xη and ∂xφ̃; the others w̃ of 16 columns each.  In the blocks of the solves, w̃ had made few
+// blocks of high order work through hundreds of columns (26×8, P = 12: 54 µs; the three launches before
+// them 21).
 __global__ void __launch_bounds__(kRecThreads) k_recover(SurfTables t, const double* __restrict__ Phi,
                                                          const double* __restrict__ eta,
                                                          const double* __restrict__ phis, double* __restrict__ w,
                                                          double* __restrict__ etax, double* __restrict__ phisx) {
   extern __shared__ double sm[];
-  const int Nx = t.Nx, P = t.P, N = t.nif, W = t.win;
+  const int Nx = t.Nx, P = t.P, N = t.nif, W = t.win, nrec = rec_blocks(Nx);
+  if ((int)blockIdx.x >= nrec) {
+    const int col = ((int)blockIdx.x - nrec) * kRecCols + (threadIdx.x >> 3);
+    wsurf_column8(t, Phi, eta, w, col < t.ncol ? col : -1, threadIdx.x & 7);
+    return;
+  }
   const int e0 = blockIdx.x * kRecElems, e1 = min(Nx, e0 + kRecElems), ne = e1 - e0;
   const int nwin = ne + 2 * W + 2;                    // elements e0 − W − 1 … e1 + W
   double* gl = sm;                                    // [2][nwin] left and right boundary rows
@@ -45,10 +52,6 @@ __global__ void __launch_bounds__(kRecThreads) k_recover(SurfTables t, const dou
     (end ? gr : gl)[fld * nwin + i] = v;
   }
   const int c0 = e0 * P, c1 = e1 * P + ((!t.periodic && e1 == Nx) ? 1 : 0);
-  for (int q0 = 0; q0 < 8 * (c1 - c0); q0 += blockDim.x) {
-    const int q = q0 + threadIdx.x, col = c0 + (q >> 3);
-    wsurf_column8(t, Phi, eta, w, col < c1 ? col : -1, q & 7);
-  }
   __syncthreads();
   const int rh = threadIdx.x >> 5;
   if (rh < 2) {
@@ -139,13 +142,14 @@ __global__ void k_rk4(int stage, int n, double dt, double* __restrict__ eta, dou
 cudaError_t launch_recover(const SurfTables& t, const double* Phi, const double* eta, const double* phis, double* w,
                            double* etax, double* phisx, cudaStream_t s) {
   const size_t smem = sizeof(double) * (4 * (kRecElems + 2 * t.win + 2) + 2 * (kRecElems + 1));
-  k_recover<<<(t.Nx + kRecElems - 1) / kRecElems, kRecThreads, smem, s>>>(t, Phi, eta, phis, w, etax, phisx);
+  const int grid = rec_blocks(t.Nx) + (t.ncol + kRecCols - 1) / kRecCols;
+  k_recover<<<grid, kRecThreads, smem, s>>>(t, Phi, eta, phis, w, etax, phisx);
   count_launch();
   return cudaGetLastError();
 }
 
 cudaError_t launch_mass1d(const SurfTables& t, const double* R, double* u0, double* u1, cudaStream_t s) {
-  k_mass1d<<<(t.Nx + kRecElems - 1) / kRecElems, kRecThreads, 0, s>>>(t, R, u0, u1);
+  k_mass1d<<<rec_blocks(t.Nx), kRecThreads, 0, s>>>(t, R, u0, u1);
   count_launch();
   return cudaGetLastError();
 }
