@@ -272,6 +272,7 @@ int do_solve(sem_mesh* m, const double* phis, double* Phi, cudaStream_t s) {
   PcgArgs a = m->pa;
   a.x = Phi;
   a.phis = phis;
+  a.start_margin = 1.0;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (m->timing) {
     CUDA_TRY(take_event(m, &e0));

@@ -1030,8 +1030,9 @@ __device__ bool finish_precondition(const DevGeom& g, Smem<P, T>& s, const Range
 // solve instead (probe), and the solve ends there; a start good enough ends before anything.  512 uneven tanks
 // (1.6 iterations a solve) 11.46 → 9.91 ms, shoal step 1515 → 1362 µs, 64×4 551 → 520, 24 Laplace
 // requests 6.34 → 5.72 ms.
-// A start is taken as the solution without an iteration only a decade below the tolerance: a good guess's
-// error is smooth, and its residual flatters it.
+// A stage's start is taken as the solution without an iteration only a decade below the tolerance
+// (PcgArgs::start_margin): an extrapolated guess's error is smooth, and its residual flatters it.  A caller's
+// start and the last potential are taken at the tolerance, without an iteration.
 constexpr double kStartMargin = 1e-2;
 template <int P, class T, class A, class TP, bool CACHE = false>
 __device__ int cg_solve(const DevGeom& g, Smem<P, T>& s, const Range& R, const Team& tm, const PcgArgs& PA,
@@ -1043,7 +1044,7 @@ __device__ int cg_solve(const DevGeom& g, Smem<P, T>& s, const Range& R, const T
   int cur = 0;
   const bool lines = use_lines<P>(g, R.e1 - R.e0);
   SEM_MARK(g, tm, TR_CG_START);
-  if (*rr_out <= kStartMargin * target) return 0;
+  if (*rr_out <= PA.start_margin * target) return 0;
   double rn = 0.0;
   cg_update<P, T, TP, CACHE>(g, s, R, tm, pv, PA.precond, V, cur, false, true, T(0), T(0), false, rn);
   if (!finish_precondition<P, T, TP, CACHE>(g, s, R, tm, PA, pv, V, s_flag, false, rn, target, red)) return -1;
@@ -1105,7 +1106,7 @@ __device__ int cg_solve(const DevGeom& g, Smem<P, T>& s, const Range& R, const T
       rr = sums[2];
       int stop = 0;
       if (!(rr == rr) || isinf(rr) || !(sums[1] == sums[1])) { atomicOr(g.status, ST_NONFINITE); stop = 1; }
-      else if (rr <= (k == 0 ? kStartMargin * target : target) || k >= max_it) stop = 1;
+      else if (rr <= (k == 0 ? PA.start_margin * target : target) || k >= max_it) stop = 1;
       if (!stop) {
         // α = γ/(δ − βγ/α_prev); thread 32 takes the next iteration's 1/γ and 1/α = den/γ
         const double gam = sums[0], del = sums[1];
@@ -1314,7 +1315,7 @@ __device__ bool solve_body(const DevGeom& g, const PcgArgs& A, const Team& tm, u
     bool stalled = false;
     while (true) {
       if (threadIdx.x == 0) {
-        int go = rr > (refinements == 0 ? kStartMargin * target : target) && iters < A.max_iter && !stalled;
+        int go = rr > (refinements == 0 ? A.start_margin * target : target) && iters < A.max_iter && !stalled;
         if (!(rr == rr) || isinf(rr)) { atomicOr(g.status, ST_NONFINITE); go = 0; }
         s_go = go;
       }
@@ -1863,7 +1864,10 @@ __device__ void stage_body(Instance& I, const Team& tm, int stage, int step, uns
   if (entry && tm.rank == 0 && threadIdx.x < 6)   // every CTA has read them
     I.hist_d[threadIdx.x] = threadIdx.x == 0 ? hm : threadIdx.x == 1 ? h1 : 0;
   // Laplace solve from the guess
-  if (threadIdx.x == 0) I.pa.phis = pin;
+  if (threadIdx.x == 0) {
+    I.pa.phis = pin;
+    I.pa.start_margin = keep ? kStartMargin : 1.0;
+  }
   __syncthreads();
   if (!solve_body<P, MIXED, CACHE>(g, I.pa, tm, smem_raw, red, s_flag)) return;
   SEM_MARK(g, tm, TR_SOLVED);

@@ -139,6 +139,7 @@ struct PcgArgs {
   float *d32, *r32, *z32, *p32a, *p32b, *q32, *edge32;
   double* part;           // reduction partials [4 slots][4 values][max grid]
   int part_stride;        // max grid
+  double start_margin;    // a start counts as the solution at this part of the target ‖r‖²
   unsigned int* bar;      // grid barrier: arrivals, exits; left at zero by every launch
   SolveRecord* rec;
   double* r64b;           // second residual buffer (double-buffered update)
