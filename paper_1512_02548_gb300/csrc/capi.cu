@@ -670,8 +670,16 @@ static int mesh_create_impl(const sem_params* pin, const double* x_edges_h, cons
     if (v >= 1 && v < m->grid) m->grid = v;
   }
 
+  const char* fz = std::getenv("SEM_FUSED_STAGE");
+  m->fused = !(fz && fz[0] == '0') && p.precond == SEM_PRECOND_SEPARABLE;
+
   Carve cv;
   const size_t nE = (size_t)Nx * nrow;
+  // Only what the mesh's own solves and steps use: the Krylov vectors of its precision, the inverse diagonal
+  // with the Jacobi preconditioner, the guess history (72 bytes a node) with the fused stages.
+  const bool mixed = p.precision == SEM_PREC_MIXED;
+  const size_t n64 = mixed ? 0 : n, n32 = mixed ? n : 0, nJ = p.precond == SEM_PRECOND_JACOBI ? n : 0,
+               nH = m->fused ? n : 0;
   // the arrays filled on the host come first: one copy uploads all of them ([0, up_end) of the block)
   const size_t o_cxz = cv.take<double>((size_t)Nx * Nz * 2), o_r2dx = cv.take<double>(Nx);
   const size_t o_h = cv.take<double>(ncol), o_hx = cv.take<double>((size_t)Nx * Q), o_dxe = cv.take<double>(Nx),
@@ -685,19 +693,20 @@ static int mesh_create_impl(const sem_params* pin, const double* x_edges_h, cons
                o_tm = cv.take<double>(N), o_tcp = cv.take<double>(N);
   const size_t up_end = cv.off;
   const size_t o_geo64 = cv.take<double>((size_t)Nx * Q * 4),
-               o_geo32 = cv.take<float>((size_t)Nx * Q * 4), o_id64 = cv.take<double>(n), o_id32 = cv.take<float>(n),
+               o_geo32 = cv.take<float>((size_t)Nx * Q * 4), o_id64 = cv.take<double>(nJ), o_id32 = cv.take<float>(nJ),
                o_status = cv.take<int>(4), o_rec = cv.take<SolveRecord>(1), o_bar = cv.take<unsigned>(4),
                o_part = cv.take<double>((size_t)16 * m->grid);
-  const size_t o_r64 = cv.take<double>(n), o_z64 = cv.take<double>(n), o_p64a = cv.take<double>(n),
-               o_p64b = cv.take<double>(n), o_q64 = cv.take<double>(n), o_q64b = cv.take<double>(n),
+  const size_t o_r64 = cv.take<double>(n), o_z64 = cv.take<double>(n64), o_p64a = cv.take<double>(n64),
+               o_p64b = cv.take<double>(n64), o_q64 = cv.take<double>(n), o_q64b = cv.take<double>(n),
                o_e64 = cv.take<double>(nE), o_e64b = cv.take<double>(nE);
-  const size_t o_d32 = cv.take<float>(n), o_r32 = cv.take<float>(n), o_z32 = cv.take<float>(n),
-               o_p32a = cv.take<float>(n), o_p32b = cv.take<float>(n), o_q32 = cv.take<float>(n),
-               o_e32 = cv.take<float>(nE);
+  const size_t o_d32 = cv.take<float>(n32), o_r32 = cv.take<float>(n32), o_z32 = cv.take<float>(n32),
+               o_p32a = cv.take<float>(n32), o_p32b = cv.take<float>(n32), o_q32 = cv.take<float>(n32),
+               o_e32 = cv.take<float>(mixed ? nE : 0);
   const size_t o_Phi = cv.take<double>(n), o_qtmp = cv.take<double>(n), o_etmp = cv.take<double>(nE);
-  const size_t o_r64b = cv.take<double>(n), o_r32b = cv.take<float>(n);
-  const size_t o_s64b = cv.take<double>(n), o_s32b = cv.take<float>(n);
-  const size_t o_uh64 = cv.take<double>((size_t)m->grid * nrow), o_uh32 = cv.take<float>((size_t)m->grid * nrow);
+  const size_t o_r64b = cv.take<double>(n64), o_r32b = cv.take<float>(n32);
+  const size_t o_s64b = cv.take<double>(n64), o_s32b = cv.take<float>(n32);
+  const size_t o_uh64 = cv.take<double>(mixed ? 0 : (size_t)m->grid * nrow),
+               o_uh32 = cv.take<float>(mixed ? (size_t)m->grid * nrow : 0);
   const size_t nEl = (size_t)nr * Nx, nIf = (size_t)nr * N;
   const size_t o_schur = cv.take<double>(nEl * 3),
                o_A32 = cv.take<float>(nEl * Pm * Pm + 1), o_Z32 = cv.take<float>(nEl * 2 * Pm + 1),
@@ -721,8 +730,8 @@ static int mesh_create_impl(const sem_params* pin, const double* x_edges_h, cons
   // written before they are read (the factor cache by every solve, the guess history by the first step of a
   // trajectory, which hist_d[0] = 0 marks): not cleared
   const size_t clear_end = cv.off;
-  const size_t o_gglob = cv.take<double>((size_t)3 * Nx * Nz * Q * Q), o_Pl = cv.take<double>(n),
-               o_H = cv.take<float>((size_t)4 * kHist * n), o_eend = cv.take<double>(ncol), o_pend = cv.take<double>(ncol);
+  const size_t o_gglob = cv.take<double>((size_t)3 * Nx * Nz * Q * Q), o_Pl = cv.take<double>(nH),
+               o_H = cv.take<float>((size_t)4 * kHist * nH), o_eend = cv.take<double>(ncol), o_pend = cv.take<double>(ncol);
   const size_t total = cv.off + 256;
   if (footprint_only) {
     *footprint_only = total;
@@ -814,7 +823,7 @@ static int mesh_create_impl(const sem_params* pin, const double* x_edges_h, cons
   a.part = D_(o_part); a.part_stride = m->grid;
   a.bar = reinterpret_cast<unsigned int*>(m->pool + o_bar);
   a.rec = m->rec;
-  a.tol = p.tol; a.inner_rtol = 1e-6; a.max_iter = p.max_iter; a.mixed = p.precision == SEM_PREC_MIXED;
+  a.tol = p.tol; a.inner_rtol = 1e-6; a.max_iter = p.max_iter; a.mixed = mixed;
   a.r64b = D_(o_r64b); a.r32b = F_(o_r32b);
   a.s64b = D_(o_s64b); a.s32b = F_(o_s32b);
   a.uh64 = D_(o_uh64); a.uh32 = F_(o_uh32);
@@ -848,8 +857,6 @@ static int mesh_create_impl(const sem_params* pin, const double* x_edges_h, cons
   t.wEP = zones ? D_(o_wEP) : nullptr;
   // the fused RK stage runs this mesh with one team of CTAs (at most its Krylov grid)
   {
-    const char* fz = std::getenv("SEM_FUSED_STAGE");
-    m->fused = !(fz && fz[0] == '0') && p.precond == SEM_PRECOND_SEPARABLE;
     m->stage_smem = stage_smem_bytes(P, nrow, Nz, chunk);
     int per_sm = 0, sms = 0;
     cudaError_t e = stage_occupancy(P, p.precision == SEM_PREC_MIXED, 0, m->stage_smem, &per_sm);
@@ -869,7 +876,6 @@ static int mesh_create_impl(const sem_params* pin, const double* x_edges_h, cons
     {
       const int Qd = P + 1;
       const int ne_max = (Nx + m->stage_team - 1) / m->stage_team;
-      const int mixed = p.precision == SEM_PREC_MIXED;
       int per2 = 0;
       const size_t smem_wide = stage_smem_bytes(P, nrow, Nz, ne_max);
       if (ne_max > chunk && smem_wide <= (size_t)kMaxDynSmem &&
