@@ -153,7 +153,7 @@ static __device__ __forceinline__ bool tile_range(const DevGeom& g, int ex0, int
 template <int P, class T>
 constexpr int tile_threads() { return sizeof(T) == 8 && (P == 7 || P == 8) ? 192 : kThreads; }
 template <int P, class T>
-constexpr int tile_ctas() { return sizeof(T) == 8 && P <= 8 ? 2 : 0; }
+constexpr int tile_ctas() { return sizeof(T) == 8 ? (P <= 4 ? 4 : P <= 8 ? 2 : 0) : 0; }
 
 // bulk_ok != 0: x is 16-byte aligned and interior tiles are staged by bulk copies.
 // NZC > 0: the layer count is the compile-time constant NZC (= g.Nz), which turns the row

@@ -2255,7 +2255,7 @@ cudaError_t launch_apply_tile_impl(int fp32, const DevGeom& g, const void* x, vo
   }
   const size_t elem = fp32 ? sizeof(float) : sizeof(double);
   // three (FP32) or two CTAs per SM (FP64, orders up to 8; beyond, only the shared-memory maximum caps the tile)
-  const size_t cap = fp32 ? kTileSmemTarget : tile_ctas<P, double>() == 2 ? (size_t)112 * 1024 : (size_t)kMaxDynSmem;
+  const size_t cap = fp32 ? kTileSmemTarget : P <= 8 ? (size_t)112 * 1024 : (size_t)kMaxDynSmem;
   int E = 16;
   while (E > 1 && apply_tile_smem<P>(E, g.nrow, g.Nz, elem) > cap) E >>= 1;
   const int Et = fp32 ? apply_tile_width(P, g.Nz) : 0;   // a measured FP32 width (autotuner), if set
