@@ -150,7 +150,6 @@ struct sem_mesh {
   int ncol = 0, nrow = 0, Pf = 0, nif = 0;
   long long n = 0;
   int grid = 0;
-  size_t smem = 0;
   unsigned char* pool = nullptr;
   size_t pool_bytes = 0;
   DevGeom g{};
@@ -175,6 +174,7 @@ struct sem_mesh {
   double hist_dt = NAN;
   unsigned int* stage_bars = nullptr;   // barrier pair of this mesh's own fused stage launch
   int stage_team = 0;
+  bool solve_wide = false;       // the stand-alone solve's launch: two CTAs per SM
   size_t stage_smem = 0;         // the mesh's own fused stage launch (with the factor cache)
   size_t stage_smem_batch = 0;   // in a batch launch (no factor cache)
   int gcache = 0;                // doubles of the factor cache in the own launch (0 = none)
@@ -279,11 +279,14 @@ int do_solve(sem_mesh* m, const double* phis, double* Phi, cudaStream_t s) {
     CUDA_TRY(take_event(m, &e1));
     CUDA_TRY(cudaEventRecord(e0, s));
   }
-  // the shape of the mesh's own fused stage launch: one pass over a CTA's columns, the factor cache
   DevGeom g = m->g;
-  g.chunk = m->own_chunk;
-  g.gcache = m->gcache;
-  CUDA_TRY(launch_pcg(g, a, m->stage_team, m->stage_smem, s));
+  if (m->solve_wide) {
+    CUDA_TRY(launch_pcg(g, a, 1, m->grid, m->stage_smem_batch, s));
+  } else {   // the shape of the mesh's own fused stage launch: one pass over a CTA's columns, the factor cache
+    g.chunk = m->own_chunk;
+    g.gcache = m->gcache;
+    CUDA_TRY(launch_pcg(g, a, 0, m->stage_team, m->stage_smem, s));
+  }
   if (m->timing) {
     CUDA_TRY(cudaEventRecord(e1, s));
     m->events.emplace_back(e0, e1);
@@ -663,7 +666,7 @@ static int mesh_create_impl(const sem_params* pin, const double* x_edges_h, cons
   sem_mesh* m = new sem_mesh;
   m->p = p; m->device = dev; m->ncol = ncol; m->nrow = nrow; m->n = n; m->Pf = p.Pf; m->nif = N;
   const int chunk = chunk_width(P, Nz);
-  cudaError_t ge = pcg_grid_size(P, Nz, nrow, Nx, chunk, p.precision == SEM_PREC_MIXED, &m->grid, &m->smem);
+  cudaError_t ge = pcg_grid_size(P, Nz, nrow, Nx, chunk, p.precision == SEM_PREC_MIXED, 1, &m->grid);
   if (ge != cudaSuccess) { delete m; return fail(SEM_ERR_CUDA, std::string("Krylov kernel occupancy: ") + cudaGetErrorString(ge)); }
   if (const char* lim = std::getenv("SEM_GRID_LIMIT")) {   // tuning/testing knob: cap the Krylov grid
     const int v = std::atoi(lim);
@@ -890,6 +893,13 @@ static int mesh_create_impl(const sem_params* pin, const double* x_edges_h, cons
         m->stage_smem = smem2;
         m->gcache = (int)need;
       }
+      // The stand-alone FP64 solve takes two CTAs per SM (128 registers) where that leaves a CTA one element column
+      // instead of two, and where the fused launch's shape needs several passes and the element-wise work
+      // outweighs the interface systems, which that shape solves faster (their ratio goes with Nz (P+1)³):
+      // 5333×4, P = 6 2033 → 1618 µs, 3030×4, P = 8 1831 → 1351, 194×16, P = 8 622 → 499; below the line 10256×2,
+      // P = 5 and 10667×8, P = 3 gain 4% and 38095×2, P = 3 would lose 44%.
+      m->solve_wide = !mixed && m->grid > m->stage_team &&
+                      (Nx <= m->grid || (m->own_chunk < ne_max && Nz * Qd * Qd * Qd >= 640));
     }
   }
   *out = m;
@@ -915,7 +925,7 @@ int sem_mesh_info(const sem_mesh* m, sem_info* info) {
   info->n_elements = m->p.Nx * m->p.Nz;
   info->P = m->p.P; info->Pf = m->Pf; info->Nx = m->p.Nx; info->Nz = m->p.Nz;
   info->periodic = m->p.periodic; info->precision = m->p.precision;
-  info->grid_ctas = m->grid;
+  info->grid_ctas = m->solve_wide ? m->grid : m->stage_team;
   info->stage_ctas = m->stage_team;
   info->device_bytes = (int64_t)m->pool_bytes;
   return SEM_OK;

@@ -176,13 +176,16 @@ cudaError_t launch_l2g(const DevGeom& g, int32_t* l2g, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t pcg_grid_size(int P, int Nz, int nrow, int Nx, int chunk, int mixed, int* grid, size_t* smem) {
-  *smem = apply_smem_bytes(P, nrow, Nz, chunk, sizeof(double));
+cudaError_t pcg_grid_size(int P, int Nz, int nrow, int Nx, int chunk, int mixed, int wide, int* grid) {
+  const size_t smem = apply_smem_bytes(P, nrow, Nz, chunk, sizeof(double));
   int dev = 0, sms = 0, per_sm = 0;
   cudaError_t e;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  SEM_DISPATCH_P(P, (e = pcg_occupancy_impl<PP>(mixed, *smem, &per_sm)));
+  // (the other build is asked too: the query opts its kernel in to the launch's shared memory)
+  SEM_DISPATCH_P(P, (e = pcg_occupancy_impl<PP>(mixed, !wide, smem, &per_sm)));
+  if (e != cudaSuccess) return e;
+  SEM_DISPATCH_P(P, (e = pcg_occupancy_impl<PP>(mixed, wide, smem, &per_sm)));
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorInvalidConfiguration;
   const long long cap = (long long)per_sm * sms, want = (Nx + chunk - 1) / chunk;
@@ -268,9 +271,9 @@ cudaError_t launch_prec_setup(const DevGeom& g, const PrecSetup& ps, cudaStream_
   return e;
 }
 
-cudaError_t launch_pcg(const DevGeom& g, const PcgArgs& a, int grid, size_t smem, cudaStream_t s) {
+cudaError_t launch_pcg(const DevGeom& g, const PcgArgs& a, int wide, int grid, size_t smem, cudaStream_t s) {
   cudaError_t e = cudaSuccess;
-  SEM_DISPATCH_P(g.P, (e = launch_pcg_impl<PP>(a.mixed, g, a, grid, smem, s)));
+  SEM_DISPATCH_P(g.P, (e = launch_pcg_impl<PP>(a.mixed, wide, g, a, grid, smem, s)));
   count_launch();
   return e;
 }

@@ -11,8 +11,8 @@ namespace semgb {
 template cudaError_t upload_tables_impl<SEM_ORDER>(const double*, const double*);
 template cudaError_t launch_geometry_impl<SEM_ORDER>(const DevGeom&, const double*, bool, cudaStream_t);
 template cudaError_t launch_apply_elem_impl<SEM_ORDER>(const DevGeom&, const double*, double*, double*, cudaStream_t);
-template cudaError_t pcg_occupancy_impl<SEM_ORDER>(int, size_t, int*);
-template cudaError_t launch_pcg_impl<SEM_ORDER>(int, const DevGeom&, const PcgArgs&, int, size_t, cudaStream_t);
+template cudaError_t pcg_occupancy_impl<SEM_ORDER>(int, int, size_t, int*);
+template cudaError_t launch_pcg_impl<SEM_ORDER>(int, int, const DevGeom&, const PcgArgs&, int, size_t, cudaStream_t);
 template cudaError_t launch_prec_setup_impl<SEM_ORDER>(const DevGeom&, const PrecSetup&, cudaStream_t);
 template cudaError_t launch_apply_tile_impl<SEM_ORDER>(int, const DevGeom&, const void*, void*, cudaStream_t);
 template cudaError_t stage_occupancy_impl<SEM_ORDER>(int, int, size_t, int*);

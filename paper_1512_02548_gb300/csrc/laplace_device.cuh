@@ -1361,16 +1361,16 @@ __device__ bool solve_body(const DevGeom& g, const PcgArgs& A, const Team& tm, u
 }
 
 // One CTA per SM with the full register file, like the mesh's own fused stage launch, with the same chunks
-// and factor cache.
-template <int P, bool MIXED>
-__global__ void __launch_bounds__(kThreads, 1) k_pcg(DevGeom g, PcgArgs A) {
+// and factor cache; WIDE: two per SM at 128 registers (FP64).
+template <int P, bool MIXED, bool WIDE = false>
+__global__ void __launch_bounds__(kThreads, WIDE ? 2 : 1) k_pcg(DevGeom g, PcgArgs A) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double red[kRedSize];
   __shared__ int s_flag[2];   // barrier result, barriers passed
   if (threadIdx.x == 0) s_flag[1] = 0;
   const Team tm{(int)blockIdx.x, (int)gridDim.x, A.bar, g.status, A.part, A.part_stride, g.bar_timeout_ns, 0};
   // testing hook: see sem_set_barrier_test
-  if (tm.rank != g.drop_rank) solve_body<P, MIXED, true>(g, A, tm, smem_raw, red, s_flag);
+  if (tm.rank != g.drop_rank) solve_body<P, MIXED, !WIDE>(g, A, tm, smem_raw, red, s_flag);
   bar_leave(tm);
 }
 
@@ -2057,20 +2057,25 @@ cudaError_t launch_apply_elem_impl(const DevGeom& g, const double* x, double* q,
 }
 
 template <int P>
-cudaError_t pcg_occupancy_impl(int mixed, size_t smem, int* per_sm) {
-  const void* fn = mixed ? (const void*)k_pcg<P, true> : (const void*)k_pcg<P, false>;
+static const void* pcg_fn(int mixed, int wide) {
+  if (mixed) return (const void*)k_pcg<P, true>;
+  return wide ? (const void*)k_pcg<P, false, true> : (const void*)k_pcg<P, false>;
+}
+
+template <int P>
+cudaError_t pcg_occupancy_impl(int mixed, int wide, size_t smem, int* per_sm) {
+  const void* fn = pcg_fn<P>(mixed, wide);
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
   if (e != cudaSuccess) return e;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, fn, kThreads, smem);
 }
 
 template <int P>
-cudaError_t launch_pcg_impl(int mixed, const DevGeom& g, const PcgArgs& a, int grid, size_t smem, cudaStream_t s) {
+cudaError_t launch_pcg_impl(int mixed, int wide, const DevGeom& g, const PcgArgs& a, int grid, size_t smem, cudaStream_t s) {
   DevGeom gg = g;
   PcgArgs aa = a;
   void* args[] = {&gg, &aa};
-  const void* fn = mixed ? (const void*)k_pcg<P, true> : (const void*)k_pcg<P, false>;
-  return cudaLaunchCooperativeKernel(fn, grid, kThreads, args, smem, s);
+  return cudaLaunchCooperativeKernel(pcg_fn<P>(mixed, wide), grid, kThreads, args, smem, s);
 }
 
 template <int P>
@@ -2152,9 +2157,9 @@ cudaError_t launch_stage_cluster_impl(int mixed, int wide, const StageArgs& a, i
   return cudaLaunchKernelExC(&cfg, stage_fn<P>(mixed, wide), args);
 }
 
-// Tiled apply (apply_tile.cuh): widest tile of at most 16 elements whose shared memory keeps
-// three CTAs per SM (FP32; the measured width where one is set) or fits at all (FP64, one CTA per
-// SM); persistent CTAs (at most the co-resident count) stride over the tiles.
+// Tiled apply (apply_tile.cuh): widest tile of at most 16 elements whose shared memory keeps three CTAs
+// per SM (FP32; the measured width where one is set), two (FP64, orders up to 8) or fits at all (FP64
+// beyond, one CTA per SM); persistent CTAs (at most the co-resident count) stride over the tiles.
 // The tensor-core FP32 kernel (apply_tc.cuh, fp32 = 3, orders 4..7) takes tiles of 64/Nz − 1
 // elements: with the recomputed left neighbour, 64 element blocks, four block pairs per warp.
 constexpr size_t kTileSmemTarget = 76 * 1024;

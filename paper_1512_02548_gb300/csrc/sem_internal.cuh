@@ -238,8 +238,8 @@ template <int P> cudaError_t launch_geometry_impl(const DevGeom& g, const double
                                                   cudaStream_t s);
 template <int P> cudaError_t launch_apply_elem_impl(const DevGeom& g, const double* x, double* q, double* edge,
                                                     cudaStream_t s);
-template <int P> cudaError_t pcg_occupancy_impl(int mixed, size_t smem, int* per_sm);
-template <int P> cudaError_t launch_pcg_impl(int mixed, const DevGeom& g, const PcgArgs& a, int grid, size_t smem,
+template <int P> cudaError_t pcg_occupancy_impl(int mixed, int wide, size_t smem, int* per_sm);
+template <int P> cudaError_t launch_pcg_impl(int mixed, int wide, const DevGeom& g, const PcgArgs& a, int grid, size_t smem,
                                              cudaStream_t s);
 template <int P> cudaError_t launch_prec_setup_impl(const DevGeom& g, const PrecSetup& ps, cudaStream_t s);
 template <int P> cudaError_t launch_apply_tile_impl(int fp32, const DevGeom& g, const void* x, void* y,
@@ -282,9 +282,9 @@ int apply_tile_width(int P, int Nz);
 // Allocation-free apply (scratch in a static device array of kNoAllocEdgeMax doubles).
 constexpr size_t kNoAllocEdgeMax = size_t(1) << 20;
 cudaError_t launch_apply_noalloc(const DevGeom& g, const double* x, double* y, cudaStream_t s);
-cudaError_t pcg_grid_size(int P, int Nz, int nrow, int Nx, int chunk, int mixed, int* grid, size_t* smem);
+cudaError_t pcg_grid_size(int P, int Nz, int nrow, int Nx, int chunk, int mixed, int wide, int* grid);
 cudaError_t launch_prec_setup(const DevGeom& g, const PrecSetup& ps, cudaStream_t s);
-cudaError_t launch_pcg(const DevGeom& g, const PcgArgs& a, int grid, size_t smem, cudaStream_t s);
+cudaError_t launch_pcg(const DevGeom& g, const PcgArgs& a, int wide, int grid, size_t smem, cudaStream_t s);
 
 // ---- launchers (kernels_surface.cu) ----
 // w̃ and the M'-projected ∂x of η and φ̃ (one kernel).
