@@ -141,7 +141,9 @@ __global__ void __launch_bounds__(ElemTile<P, NZ>::threads, ElemTile<P, NZ>::cta
     float yv[Q][Q];                              // [a][b]: x even-odd sums of the result, then the result
     if (on) {
       const double2 cz = Cs[el * NZ + l];
-      const float c0 = (float)cz.x, c1 = (float)cz.y;
+      float c0, c0l, c1, c1l;
+      split_ratio(cz.x, c0, c0l);
+      split_ratio(cz.y, c1, c1l);
       float u[Q][Q];
       const float* Xe = X + el * L::se + l * P;
 #pragma unroll
@@ -149,27 +151,27 @@ __global__ void __launch_bounds__(ElemTile<P, NZ>::threads, ElemTile<P, NZ>::cta
 #pragma unroll
         for (int b = 0; b < Q; ++b) u[a][b] = Xe[(a < P ? a * nrow : L::se) + b];
 #pragma unroll
-      for (int i = 0; i < h; ++i)                // u[i] ← u_i + u_{P−i}, u[P−i] ← u_i − u_{P−i}
+      for (int i = 0; i < h; ++i)                // u[i], u[P−i] ← e_i − 2 u_mid, o_i of the x-lines (eo_diff)
 #pragma unroll
         for (int b = 0; b < Q; ++b) {
-          const float p = u[i][b], q = u[P - i][b];
-          u[i][b] = p + q;
+          const float p = u[i][b], q = u[P - i][b], m = u[h][b];
           u[P - i][b] = p - q;
+          u[i][b] = P - i == h ? p - q : (p - m) + (q - m);
         }
 #pragma unroll
       for (int a = 0; a < Q; ++a)
 #pragma unroll
         for (int b = 0; b < Q; ++b) yv[a][b] = 0.f;
-      const float* w = c_w32 + w_off(P);
+      const float* w = c_eo.w32s;
       // F1/w_a and F2/w_a of one column from u_r and u_t
       auto flux = [&](int a, const float (&ur)[Q], const float (&ut)[Q], float (&F1)[Q], float (&F2)[Q]) {
         const float4 q = Gs[el * Q + a];
-        const float g11 = c0 * q.x, g22 = c1 * q.y;
+        const float g11 = fmaf(c0, q.x, c0l * q.x), g22 = fmaf(c1, q.y, c1l * q.y);
 #pragma unroll
         for (int b = 0; b < Q; ++b) {
           const float K12 = fmaf(-sg[b], q.w, q.z);
-          F1[b] = w[b] * fmaf(K12, ut[b], g11 * ur[b]);
-          F2[b] = fmaf(K12, ur[b], g22 * fmaf(K12, K12, 1.f) * ut[b]);
+          F1[b] = w[b] * fmaf(g11, ur[b], K12 * ut[b]);   // the large products are not rounded by themselves
+          F2[b] = fmaf(g22 * fmaf(K12, K12, 1.f), ut[b], K12 * ur[b]);
         }
       };
 #pragma unroll
@@ -177,20 +179,23 @@ __global__ void __launch_bounds__(ElemTile<P, NZ>::threads, ElemTile<P, NZ>::cta
         float r1[Q], r2[Q], t1[Q], t2[Q], F1a[Q], F2a[Q], F1b[Q], F2b[Q];
 #pragma unroll
         for (int b = 0; b < Q; ++b) {
-          float S = c_eo.D32.O[i * eo_stride(Q)] * u[P][b], V = c_eo.D32.E[i * eo_stride(Q)] * u[0][b];
+          float S = c_eo.D32s.O[i * eo_stride(Q)] * u[P][b], V = c_eo.D32s.E[i * eo_stride(Q)] * u[0][b];
 #pragma unroll
           for (int j = 1; j < h; ++j) {
-            S = fmaf(c_eo.D32.O[i * eo_stride(Q) + j], u[P - j][b], S);
-            V = fmaf(c_eo.D32.E[i * eo_stride(Q) + j], u[j][b], V);
+            S = fmaf(c_eo.D32s.O[i * eo_stride(Q) + j], u[P - j][b], S);
+            V = fmaf(c_eo.D32s.E[i * eo_stride(Q) + j], u[j][b], V);
           }
-          if constexpr (Q % 2) V = fmaf(c_eo.D32.C[i], u[h][b], V);
           r1[b] = S + V;
           r2[b] = S - V;
         }
-        eo_line<Q, float>(c_eo.Dh32, u[i], t1);      // ½D of the sum and of the difference
-        eo_line<Q, float>(c_eo.Dh32, u[P - i], t2);
+        float ua[Q], ub[Q];                          // the two columns again, from the staging buffer
 #pragma unroll
-        for (int b = 0; b < Q; ++b) { const float p = t1[b], q = t2[b]; t1[b] = p + q; t2[b] = p - q; }
+        for (int b = 0; b < Q; ++b) {
+          ua[b] = Xe[i * nrow + b];
+          ub[b] = Xe[(P - i < P ? (P - i) * nrow : L::se) + b];
+        }
+        eo_diff<Q, float>(c_eo.D32s, ua, t1);
+        eo_diff<Q, float>(c_eo.D32s, ub, t2);
         flux(i, r1, t1, F1a, F2a);
         flux(P - i, r2, t2, F1b, F2b);
 #pragma unroll
@@ -198,16 +203,16 @@ __global__ void __launch_bounds__(ElemTile<P, NZ>::threads, ElemTile<P, NZ>::cta
           const float fe = F1a[b] + F1b[b], fo = F1a[b] - F1b[b];
 #pragma unroll
           for (int c = 0; c < h; ++c) {
-            yv[c][b] = fmaf(c_eo.H32.O[c * eo_stride(Q) + i], fo, yv[c][b]);          // S_c
-            yv[P - c][b] = fmaf(c_eo.H32.E[c * eo_stride(Q) + i], fe, yv[P - c][b]);  // T_c
+            yv[c][b] = fmaf(c_eo.H32s.O[c * eo_stride(Q) + i], fo, yv[c][b]);          // S_c
+            yv[P - c][b] = fmaf(c_eo.H32s.E[c * eo_stride(Q) + i], fe, yv[P - c][b]);  // T_c
           }
-          if constexpr (Q % 2) yv[h][b] = fmaf(c_eo.H32.R[i], fo, yv[h][b]);
+          if constexpr (Q % 2) yv[h][b] = fmaf(c_eo.H32s.R[i], fo, yv[h][b]);
           const float p = F2a[b], q = F2b[b];
           F2a[b] = p + q;
           F2b[b] = p - q;
         }
-        eo_line<Q, float>(c_eo.H32, F2a, t1);
-        eo_line<Q, float>(c_eo.H32, F2b, t2);
+        eo_line<Q, float>(c_eo.H32s, F2a, t1);
+        eo_line<Q, float>(c_eo.H32s, F2b, t2);
         const float wh = 0.5f * w[i];
 #pragma unroll
         for (int b = 0; b < Q; ++b) { yv[i][b] = fmaf(wh, t1[b], yv[i][b]); yv[P - i][b] = fmaf(wh, t2[b], yv[P - i][b]); }
@@ -216,17 +221,17 @@ __global__ void __launch_bounds__(ElemTile<P, NZ>::threads, ElemTile<P, NZ>::cta
         float r[Q], t[Q], F1[Q], F2[Q];
 #pragma unroll
         for (int b = 0; b < Q; ++b) {
-          r[b] = c_eo.D32.R[0] * u[P][b];
+          r[b] = c_eo.D32s.R[0] * u[P][b];
 #pragma unroll
-          for (int j = 1; j < h; ++j) r[b] = fmaf(c_eo.D32.R[j], u[P - j][b], r[b]);
+          for (int j = 1; j < h; ++j) r[b] = fmaf(c_eo.D32s.R[j], u[P - j][b], r[b]);
         }
-        eo_line<Q, float>(c_eo.D32, u[h], t);
+        eo_diff<Q, float>(c_eo.D32s, u[h], t);
         flux(h, r, t, F1, F2);
-        eo_line<Q, float>(c_eo.H32, F2, t);
+        eo_line<Q, float>(c_eo.H32s, F2, t);
 #pragma unroll
         for (int b = 0; b < Q; ++b) {
 #pragma unroll
-          for (int c = 0; c < h; ++c) yv[P - c][b] = fmaf(c_eo.H32.C[c], F1[b], yv[P - c][b]);
+          for (int c = 0; c < h; ++c) yv[P - c][b] = fmaf(c_eo.H32s.C[c], F1[b], yv[P - c][b]);
           yv[h][b] = fmaf(w[h], t[b], yv[h][b]);
         }
       }

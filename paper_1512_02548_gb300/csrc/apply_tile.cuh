@@ -13,12 +13,9 @@
 // while the current one is computed.  A tile's values are one contiguous range of x
 // (columns are stored back to back); the copy starts at the 16-byte boundary below the
 // range and the tile is read at the resulting offset.  Tiles whose range wraps around the
-// periodic end, or whose rounded range would pass the end of x, are staged with plain loads.
+// periodic end, or whose rounded range would pass the end of x, are staged value by value (cp.async).
 //
 // Per tile, with the tile's nodal values staged in shared memory:
-// Every contraction is taken in its even-odd form (even_odd.cuh): FP64, which holds the narrow FP64 pipe,
-// needs about 42 operations per node instead of 54, and two CTAs per SM cover each other's barriers:
-// 30011×2, P = 7: 424 → 320 µs; 8 M nodes, P = 4..10: 20–40% less.
 //   1. x-lines (element e, layer l, row b): u_r(a) = Σ_c D_ac u(c,b) for all a, in registers;
 //   2. σ-lines (e, l, column a): u_t(b) = Σ_c D_bc u(a,c); the geometric factors of column a
 //      (d, 1/d, ∂xh, ∂xd) and the layer ratios give
@@ -29,6 +26,9 @@
 //   4. the contributions are stored into the tile's nodes; the nodes shared between layers
 //      and between elements are completed by two small fix-up sweeps in a fixed order (no
 //      atomics), and the tile's own columns are written as −sum with contiguous stores.
+// Every contraction is taken in its even-odd form (even_odd.cuh): FP64, which holds the narrow FP64 pipe,
+// needs about 43 operations per node instead of 54, and two CTAs per SM cover each other's barriers:
+// 30011×2, P = 7: 424 → 330 µs; 4 M nodes, P = 4..12: 10–34% less.
 // All sums have a fixed order: results are bitwise reproducible.
 #pragma once
 
@@ -118,7 +118,7 @@ struct TileLayout {
   // buffers, the line buffers and the tile's geometry
   __host__ __device__ size_t bytes(int nrow, int Nz, int elem) const {
     return 16 + (size_t)elem * (2 * (size_t)xbuf + 3 * (size_t)nline + (size_t)en_max * Q * 4 +
-                                (size_t)en_max * Nz * 2 + nrow + Q + 2 * (size_t)en_max * Nz * Q);
+                                (size_t)en_max * Nz * (elem == 4 ? 4 : 2) + nrow + Q + 2 * (size_t)en_max * Nz * Q);
   }
   // the same for the tensor-core kernel (FP32): the tile's node buffer and `scratch` floats per
   // warp in place of the three line buffers
@@ -147,9 +147,30 @@ static __device__ __forceinline__ bool tile_range(const DevGeom& g, int ex0, int
   return true;
 }
 
+// A ratio c > 0 as hi + lo in FP32.  Rounded, it would put the same error on every node of the element; its low
+// bits cost an operation per column (from the words of c: conversions back and forth hold the FP64 pipe).
+static __device__ __forceinline__ void split_ratio(double c, float& hi, float& lo) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(c);
+  const int e = (int)(b >> 52) - 896;            // FP32 exponent field
+  if (e > 52 && e < 255) {
+    hi = __uint_as_float(((unsigned)e << 23) | ((unsigned)(b >> 29) & 0x7fffffu));
+    lo = (float)((unsigned)b & 0x1fffffffu) * __uint_as_float((unsigned)(e - 52) << 23);
+  } else {
+    hi = (float)c;
+    lo = 0.f;
+  }
+}
+
+// Weights that go with eo_Ds and eo_Hs.
+template <class T, int P> __device__ __forceinline__ const T* eo_ws() {
+  if constexpr (sizeof(T) == 8) return CT<T>::w() + w_off(P);
+  else return c_eo.w32s;
+}
+
 // FP64: two CTAs per SM, so that one CTA's FP64 work covers the other's barriers and staging: of 256
-// threads at 128 registers up to order 6, of 192 threads at 168 registers for orders 7 and 8 (fewer
-// would spill); one CTA of 256 beyond.
+// threads at 128 registers for orders 5 and 6, of 192 threads at 168 registers for 7 and 8 (fewer
+// would spill); one CTA of 256 beyond.  Orders up to 4 have little work between barriers and take four at 64
+// registers (three at 80: 666667×1, P = 2 488 µs, four 396; 8333×1, P = 3 18.7 and 16.3).
 template <int P, class T>
 constexpr int tile_threads() { return sizeof(T) == 8 && (P == 7 || P == 8) ? 192 : kThreads; }
 template <int P, class T>
@@ -176,13 +197,14 @@ __global__ void __launch_bounds__(tile_threads<P, T>(), (sizeof(T) == 4 && P == 
   T* Fs = Ur + L.nline;                     // [en][Nz][Q b][QP a] F1
   T* Ys = Fs + L.nline;                     // [en][Nz][Q b][QP a] σ part of the transpose
   T* Gs = Ys + L.nline;                     // [en][Q][4] d, 1/d, ∂xh, ∂xd
-  T* Cs = Gs + (size_t)L.en_max * Q * 4;    // [en][Nz][2] Δσ/Δx, Δx/Δσ
-  T* Ss = Cs + (size_t)L.en_max * Nz * 2;   // [nrow] σ
+  constexpr int CS = sizeof(T) == 4 ? 4 : 2;
+  T* Cs = Gs + (size_t)L.en_max * Q * 4;    // [en][Nz][CS] Δσ/Δx, Δx/Δσ (FP32: two parts each)
+  T* Ss = Cs + (size_t)L.en_max * Nz * CS;  // [nrow] σ
   T* Ws = Ss + nrow;                        // [Q] GLL weights (indexed per thread)
   T* Rrow = Ws + Q;                         // [en][Nz][Q] top-row (b = P) contributions, a < P
   T* Ccol = Rrow + (size_t)L.en_max * Nz * Q;   // [en][Nz][Q] right-column (a = P) contributions
   __shared__ int s_ok;
-  const T* w = CT<T>::w() + w_off(P);       // compile-time indices only: constant operands
+  const T* w = eo_ws<T, P>();               // compile-time indices only: constant operands
   const T* geo = geo_ptr<T>(g);
   for (int t = threadIdx.x; t < nrow; t += blockDim.x) Ss[t] = (T)g.sig[t];
   for (int t = threadIdx.x; t < Q; t += blockDim.x) Ws[t] = w[t];
@@ -265,8 +287,13 @@ __global__ void __launch_bounds__(tile_threads<P, T>(), (sizeof(T) == 4 && P == 
       int ge = ex0 - 1 + e;
       if (ge < 0) ge = g.periodic ? ge + Nx : 0;
       const double* cz = g.cxz + ((size_t)ge * Nz + l) * 2;
-      Cs[2 * t] = (T)cz[0];
-      Cs[2 * t + 1] = (T)cz[1];
+      if constexpr (CS == 4) {
+        split_ratio(cz[0], Cs[4 * t], Cs[4 * t + 1]);
+        split_ratio(cz[1], Cs[4 * t + 2], Cs[4 * t + 3]);
+      } else {
+        Cs[2 * t] = cz[0];
+        Cs[2 * t + 1] = cz[1];
+      }
     }
     __syncthreads();
     if (!s_ok) break;                            // a copy did not complete: stop (status set below)
@@ -282,7 +309,7 @@ __global__ void __launch_bounds__(tile_threads<P, T>(), (sizeof(T) == 4 && P == 
       for (int c = 0; c < Q; ++c) u[c] = Xl[c * nrow];
       T* out = Ur + (e * Nz + l) * BS + bb * QP;
       T r[Q];
-      eo_line<Q, T>(eo_D<T>(), u, r);
+      eo_diff<Q, T>(eo_Ds<T>(), u, r);
 #pragma unroll
       for (int a = 0; a < Q; ++a) out[a] = r[a];
     }
@@ -297,22 +324,28 @@ __global__ void __launch_bounds__(tile_threads<P, T>(), (sizeof(T) == 4 && P == 
 #pragma unroll
       for (int c = 0; c < Q; ++c) u[c] = Xl[c];
       const T* gq = Gs + (e * Q + a) * 4;
-      const T c0 = Cs[2 * (e * Nz + l)], c1 = Cs[2 * (e * Nz + l) + 1];
+      const T* cs = Cs + CS * (e * Nz + l);
       const T wa = Ws[a], hx = gq[2], dxd = gq[3];
-      const T g11 = c0 * gq[0];                  // Δσ/Δx d
-      const T g22 = c1 * gq[1];                  // Δx/Δσ /d
+      T g11, g22;                                // Δσ/Δx d, Δx/Δσ /d
+      if constexpr (CS == 4) {
+        g11 = fmx(cs[0], gq[0], cs[1] * gq[0]);
+        g22 = fmx(cs[2], gq[1], cs[3] * gq[1]);
+      } else {
+        g11 = cs[0] * gq[0];
+        g22 = cs[1] * gq[1];
+      }
       const T* sg = Ss + l * P;
       const int base = (e * Nz + l) * BS;
       T ut[Q], f2[Q];
-      eo_line<Q, T>(eo_D<T>(), u, ut);
+      eo_diff<Q, T>(eo_Ds<T>(), u, ut);
 #pragma unroll
       for (int bb = 0; bb < Q; ++bb) {           // F1/w_a and F2/(w_a w_b): the weights are in the tables of H
         const T ur = Ur[base + bb * QP + a];
         const T K12 = fmx(-sg[bb], dxd, hx);
         Fs[base + bb * QP + a] = w[bb] * fmx(g11, ur, K12 * ut[bb]);
-        f2[bb] = fmx(K12, ur, g22 * fmx(K12, K12, T(1)) * ut[bb]);
+        f2[bb] = fmx(g22 * fmx(K12, K12, T(1)), ut[bb], K12 * ur);
       }
-      eo_line<Q, T>(eo_H<T>(), f2, ut);
+      eo_line<Q, T>(eo_Hs<T>(), f2, ut);
 #pragma unroll
       for (int bb = 0; bb < Q; ++bb) Ys[base + bb * QP + a] = wa * ut[bb];
     }
@@ -336,7 +369,7 @@ __global__ void __launch_bounds__(tile_threads<P, T>(), (sizeof(T) == 4 && P == 
       const bool top = bb == P && l < Nz - 1;   // row shared with the layer above
       T* yn = Yt + (e * P) * nrow + l * P + bb;
       T y1[Q];
-      eo_line<Q, T>(eo_H<T>(), f1, y1);
+      eo_line<Q, T>(eo_Hs<T>(), f1, y1);
 #pragma unroll
       for (int a = 0; a < Q; ++a) {
         const T s = Ys[row + a] + y1[a];

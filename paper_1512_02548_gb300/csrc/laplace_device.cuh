@@ -390,7 +390,7 @@ __device__ __forceinline__ T apply_element_lines(const DevGeom& g, Smem<P, T>& s
     T u[Q], r[Q];
 #pragma unroll
     for (int c = 0; c < Q; ++c) u[c] = x[c * nrow];
-    eo_line<Q, T>(eo_D<T>(), u, r);
+    eo_diff<Q, T>(eo_D<T>(), u, r);
 #pragma unroll
     for (int a = 0; a < Q; ++a) s.Y[t * QP + a] = r[a];
   }
@@ -404,7 +404,7 @@ __device__ __forceinline__ T apply_element_lines(const DevGeom& g, Smem<P, T>& s
     T u[Q], ut[Q], f[Q];
 #pragma unroll
     for (int c = 0; c < Q; ++c) u[c] = x[c];
-    eo_line<Q, T>(eo_D<T>(), u, ut);
+    eo_diff<Q, T>(eo_D<T>(), u, ut);
     const double* gl = gc ? gc + (size_t)el * 3 * QQ + a : nullptr;
     T* F = s.F1 + (size_t)el * Q * QP + a;
 #pragma unroll
@@ -2025,8 +2025,7 @@ cudaError_t upload_tables_impl(const double* D64, const double* w64) {
   fill_eo<P>(eo.T32, Dt, 1.0);
   fill_eo<P>(eo.H64, H, 1.0);
   fill_eo<P>(eo.D32, D, 1.0);
-  fill_eo<P>(eo.Dh32, D, 0.5);
-  fill_eo<P>(eo.H32, H, 1.0);
+  fill_scaled<P>(eo, D, H, w);
   if ((e = cudaMemcpyToSymbol(c_eo, &eo, sizeof(eo))) != cudaSuccess) return e;
   return cudaMemcpyToSymbol(c_w32, w32, sizeof(float) * kWTotal);
 }
