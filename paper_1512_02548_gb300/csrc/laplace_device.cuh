@@ -1501,12 +1501,11 @@ __global__ void __launch_bounds__(kPrecModesPerBlock) k_prec_elem(DevGeom g, Pre
 // One warp per mode: interface tridiagonal d_j = S00(j) + S11(j−1), e_j = S01(j) and its Thomas
 // pivots.  The pivot recurrence m_j = 1/(d_j − e_{j−1}² m_{j−1}) runs on lane 0 in FP32 from
 // shared memory (a sequential FP64 chain costs ~64 cycles per instruction on this part); the
-// FP64 factors are taken from those pivots, m⁶⁴ = m³², c' = e m, which makes them the exact
-// LDLᵀ factors of a symmetric tridiagonal within FP32 of the true one.  The Sherman–Morrison
-// vector T'⁻¹u of the periodic closure (γ = −d_0, u = (γ,0,…,0,e_{N−1}), v = (1,0,…,0,
-// e_{N−1}/γ)) is then solved with the warp-parallel tridiagonal solver and the same factors,
-// once in FP64 and once in FP32.  Staged in shared memory when 3·nif values fit, otherwise the
-// recurrence reads and writes the destination arrays directly.
+// multipliers are c' = e m of those pivots, the LDLᵀ factors of a symmetric tridiagonal within FP32 of the
+// true one.  The Sherman–Morrison vector T'⁻¹u of the periodic closure (γ = −d_0, u = (γ,0,…,0,e_{N−1}),
+// v = (1,0,…,0, e_{N−1}/γ)) is then solved with the warp-parallel tridiagonal solver and the same factors,
+// in FP32.  Staged in shared memory when 2·nif values fit, otherwise the recurrence reads and writes the
+// destination arrays directly.
 // `stage_sm`: 2·nif floats of shared memory, or nullptr to run the recurrence on the
 // destination arrays.  Called by one full warp.
 static __device__ void prec_tri_mode(const DevGeom& g, const PrecSetup& ps, int k, float* stage_sm) {
@@ -1534,8 +1533,8 @@ static __device__ void prec_tri_mode(const DevGeom& g, const PrecSetup& ps, int 
       dd[0] = (float)(2.0 * (sc[0] + sc[(Nx - 1) * 3 + 2]));
       dd[N - 1] = (float)((double)dd[N - 1] - corner * corner / gamma);
     }
-    // one lane's chain m_j = 1/(d_j − e_{j−1} c'_{j−1}): the reciprocal by the special function unit, the
-    // next eight values loaded while eight are worked off (80 → 25 ns a step)
+    // one lane's chain m_j = 1/(d_j − e_{j−1} c'_{j−1}), the next eight values loaded while eight are worked off
+    // (a correctly rounded reciprocal: the closure of a nearly singular lowest mode magnifies what differs here)
     constexpr int B = 8;
     float cp_prev = 0.f, e_prev = 0.f, dn[B], en[B];
 #pragma unroll
@@ -1552,7 +1551,7 @@ static __device__ void prec_tri_mode(const DevGeom& g, const PrecSetup& ps, int 
 #pragma unroll
       for (int q = 0; q < B; ++q)
         if (j0 + q < N) {
-          const float m = __fdividef(1.f, fmaf(-e_prev, cp_prev, dq[q]));
+          const float m = 1.f / fmaf(-e_prev, cp_prev, dq[q]);
           dd[j0 + q] = m;            // pivots overwrite the diagonal
           cp_prev = eq[q] * m;
           e_prev = eq[q];
@@ -1679,7 +1678,7 @@ static __device__ void prec_tri_mode_cta(const DevGeom& g, const PrecSetup& ps, 
   }
   __syncthreads();                                  // every chunk has read its diagonal
   for (int j = j0; j < j1; ++j) {
-    const float m = __fdividef(1.f, j == 0 ? tm32[0] : fmaf(-e_prev, cp_prev, tm32[j]));
+    const float m = 1.f / (j == 0 ? tm32[0] : fmaf(-e_prev, cp_prev, tm32[j]));
     const float e = te32[j];
     tm32[j] = m;
     tcp32[j] = e * m;
