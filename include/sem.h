@@ -171,11 +171,12 @@ int sem_laplace_apply(sem_mesh* m, const double* x_d, double* y_d, void* stream)
  * with the FP32 copy of the geometry of the last sem_update_geometry.  One kernel, tiles of
  * consecutive x-elements with the element left of each tile recomputed, so every output
  * column is complete in one CTA and written once; uses no workspace.  Orders up to 8 with up to
- * four layers take one element per thread (7 and 8 from a few thousand elements on), others
+ * four layers take one element per thread from a size on that depends on order and layers, others
  * line passes through shared memory.  x_d, y_d: device,
  * float, n values, must not overlap.  The environment variable SEM_APPLY_F32=tc selects, for
  * orders 4..7, a kernel whose element contractions run on the tensor cores (TF32 products
- * split three ways for FP32 accuracy; same result up to rounding, and slower on GB300). */
+ * split three ways for FP32 accuracy; same result up to rounding, and slower on GB300); line and
+ * elem select one of the two others at every size that it serves. */
 int sem_laplace_apply_f32(const sem_mesh* m, const float* x_d, float* y_d, void* stream);
 
 /* Allocation-free form of sem_laplace_apply (the paper has no counterpart; this is a
@@ -318,7 +319,7 @@ int sem_get_batch_tuning(sem_batch_tuning* t);
 /* Tile width (elements per tile, 1..16) of the FP32 apply by line passes (sem_laplace_apply_f32 where it
  * does not take one element per thread) for order P and Nz layers, as measured by the autotuner; 0 restores the default (the widest
  * tile up to 16 that keeps three CTAs per SM).  The FP64 apply takes the widest tile up to 16 that
- * fits in shared memory.  Process-wide. */
+ * leaves room for two CTAs per SM (orders above 8: that fits in shared memory).  Process-wide. */
 int sem_set_apply_tile_width(int P, int Nz, int E);
 
 /* Per-instance result of the last sem_batch_rk4_step or sem_batch_laplace_solve:

@@ -11,9 +11,11 @@ It measures, with CUDA events on the launching stream,
   tuned on), for every candidate of the batch planning parameters of ``sem_set_batch_tuning``:
   the cluster team share, the largest cluster and the group size up to which the one-CTA-per-SM
   build is used; the candidate with the smallest summed step time wins;
-* the FP32 tiled apply on a long periodic tank of about 9.8 M nodes (above the L2, flushed before
-  each timed apply) for every order P = 2..12, layer count Nz = 1, 2, 4 and tile width E = 1..16
-  that fits in shared memory; the fastest width per (P, Nz) wins (the FP64 apply keeps its rule);
+* the FP32 apply by line passes on a long periodic tank, the L2 flushed before each timed apply, for
+  every order P = 5..12, layer count Nz = 1, 2, 4 and tile width E = 1..16 that fits in shared memory;
+  the fastest width per (P, Nz) wins (the FP64 apply keeps its rule).  Orders 5 and 6 are measured at
+  about 0.6 M nodes, the largest size that the line passes serve (beyond, one element per thread does, which
+  has no width; orders up to 4 are left out, they hardly ever take line passes), higher ones at 9.8 M;
 
 and writes the winners with every measurement to ``tuning.json`` next to this file (or PATH);
 ``--apply-only`` re-measures the tile widths alone and keeps the file's batch section.
@@ -127,18 +129,30 @@ def tune_batch(dev, count: int = 512, seed: int = 1, steps: int = 3, quick: bool
     return {k: best[k] for k in ("cluster_share", "max_cluster", "narrow_max", "plan")}, rows
 
 
-def tune_apply(dev, nodes: float = 9.8e6, reps: int = 7, quick: bool = False):
-    """FP32 tile widths on long tanks of about `nodes` nodes (x and y above the L2), the L2 flushed
-    before each timed apply, median of `reps`."""
+def tune_apply(dev, nodes: float = 9.8e6, nodes_low: float = 6e5, reps: int = 7, quick: bool = False):
+    """FP32 tile widths of the line passes on long tanks of about `nodes` nodes (x and y above the L2), or
+    `nodes_low` for orders 5 and 6, the L2 flushed before each timed apply, median of `reps`."""
+    old = os.environ.get("SEM_APPLY_F32")
+    os.environ["SEM_APPLY_F32"] = "line"
+    try:
+        return _tune_line_passes(dev, nodes, nodes_low, reps, quick)
+    finally:
+        if old is None:
+            del os.environ["SEM_APPLY_F32"]
+        else:
+            os.environ["SEM_APPLY_F32"] = old
+
+
+def _tune_line_passes(dev, nodes, nodes_low, reps, quick):
     import torch
     from . import Mesh, set_apply_tile_width
     from sem_workloads import roofline_tank
     winners, rows = {}, []
     flush = torch.empty(64 << 20, dtype=torch.float32, device=dev)   # 256 MB, above the L2
-    orders = (4, 6, 8) if quick else range(2, 13)
+    orders = (6, 8, 10) if quick else range(5, 13)
     for P in orders:
         for Nz in (1, 2, 4):
-            Nx = max(64, int(nodes / (P * (Nz * P + 1))))
+            Nx = max(64, int((nodes_low if P <= 6 else nodes) / (P * (Nz * P + 1))))
             wl = roofline_tank(Nx=Nx, Nz=Nz, P=P)
             mesh = Mesh.from_workload(wl)
             mesh.update_geometry(torch.zeros(wl.ncol, dtype=torch.float64, device=dev))
@@ -185,14 +199,14 @@ def main():
     load_library()
     dev = torch.device("cuda", 0)
     t0 = time.time()
+    now = batch_when = time.strftime("%Y-%m-%dT%H:%M:%SZ", time.gmtime())
     if args.apply_only:
         old = json.load(open(args.out))
-        batch, batch_rows = old["batch"], old["measured"]["batch"]
+        batch, batch_rows, batch_when = old["batch"], old["measured"]["batch"], old.get("batch_when", old["when"])
     else:
         batch, batch_rows = tune_batch(dev, quick=args.quick)
     tiles, tile_rows = tune_apply(dev, quick=args.quick)
-    out = {"device": torch.cuda.get_device_name(0), "when": time.strftime("%Y-%m-%dT%H:%M:%SZ", time.gmtime()),
-           "batch": batch, "apply_tile_width": tiles,
+    out = {"device": torch.cuda.get_device_name(0), "when": now, "batch_when": batch_when, "batch": batch, "apply_tile_width": tiles,
            "measured": {"batch": batch_rows, "apply_tile": tile_rows,
                         "batch_workload": "512 uneven periodic tanks, seed 1, drawn like the benchmark batch (seed 0)",
                         "seconds": time.time() - t0}}

@@ -10,9 +10,9 @@ namespace semgb {
 // The line-pass kernel (k_apply_tile) spends 142 instructions per node, two thirds of them moving
 // lines between its three passes through shared memory.  Here a thread loads the (P+1)² values of its
 // element once, keeps every intermediate in registers, and exchanges only the top row and the right
-// column with its neighbours: about 43 FP32 operations per node, FP32-issue bound (58% of the issue slots
-// at 12 warps an SM).  65536×4, P = 6: 63.5 → 30.5 µs (2.6 TB/s of x and y); 8 M nodes of P = 3..8: 51–138 →
-// 25–62 µs.
+// column with its neighbours: about 43 FP32 operations per node.  What bounds it is the latency of a thread's long
+// chains at 12 warps an SM (6 at order 8, 1 or 2 CTAs by registers and shared memory), 58% of the issue slots used.
+// 65536×4, P = 6: 63.5 → 30.5 µs (2.6 TB/s of x and y); 8 M nodes of P = 3..8: 51–138 → 25–62 µs.
 // A warp holds 32 consecutive elements of one layer; a CTA holds all layers of 32·G elements, the first
 // of which is the element left of its tile, recomputed for the tile's first column.  x is staged by bulk
 // copies, double-buffered as in k_apply_tile; y goes through the same buffer and leaves in contiguous
@@ -23,8 +23,6 @@ struct ElemTile {
   static constexpr int G = NZ == 1 ? 4 : (NZ <= 3 ? 2 : 1);   // groups of 32 elements
   static constexpr int en = 32 * G, E = en - 1;               // elements computed, owned
   static constexpr int threads = 32 * NZ * G;
-  // CTAs per SM: 168 registers up to order 6, else 255
-  static constexpr int ctas = P <= 6 ? (threads <= 128 ? 3 : 2) : (threads <= 128 ? 2 : 1);
   // Floats between elements in the staging buffer.  Lanes read their elements at this stride: where it
   // would be a multiple of 8 words (8- or 16-way bank conflicts), the elements, then whole 16-byte
   // multiples, are copied one by one with 4 words between them (tanks of P = 5, three
@@ -35,6 +33,10 @@ struct ElemTile {
   static constexpr int xbuf = ((en * se + nrow + 8 + 3) / 4) * 4;
   static constexpr int gbuf = 4 * en * Q, cbuf = 4 * en * NZ;   // floats: geometry, layer ratios (FP64)
   static constexpr size_t smem = 16 + 4 * (size_t)(2 * (xbuf + gbuf + cbuf) + NZ * (P + Q) * en);
+  // CTAs per SM: 168 registers up to order 6, else 255, and as many as the shared memory holds (6, 1: two, 8, 1: one)
+  static constexpr int reg_ctas = P <= 6 ? (threads <= 128 ? 3 : 2) : (threads <= 128 ? 2 : 1);
+  static constexpr int smem_ctas = (int)((size_t)228 * 1024 / (smem + 1024 + 16));
+  static constexpr int ctas = reg_ctas < smem_ctas ? reg_ctas : smem_ctas;
 };
 
 template <int P, int NZ>

@@ -869,6 +869,7 @@ static int mesh_create_impl(const sem_params* pin, const double* x_edges_h, cons
       delete m;
       return fail(SEM_ERR_CUDA, "fused stage kernel does not fit on this device");
     }
+    g.sms = sms;
     m->stage_team = std::min(m->grid, per_sm * sms);
     m->stage_smem_batch = m->stage_smem;
     m->own_chunk = chunk;
@@ -960,10 +961,11 @@ int sem_laplace_apply(sem_mesh* m, const double* x_d, double* y_d, void* stream)
 int sem_laplace_apply_f32(const sem_mesh* m, const float* x_d, float* y_d, void* stream) {
   if (!m || !x_d || !y_d || x_d == y_d) return fail(SEM_ERR_INVALID_ARG, "bad pointer");
   DeviceGuard dg(m->device);
-  // "tc": the tensor-core kernel for orders 4..7 (measured slower than the CUDA-core kernel on
-  // GB300; kept for comparison), else the CUDA-core kernel
+  // "tc": the tensor-core kernel for orders 4..7 (measured slower than the CUDA-core kernels on
+  // GB300; kept for comparison); "line", "elem": one of the CUDA-core kernels at every size it serves, for tests
   const char* k = std::getenv("SEM_APPLY_F32");
-  CUDA_TRY(launch_apply_tile(k && std::strcmp(k, "tc") == 0 ? 3 : 1, m->g, x_d, y_d, (cudaStream_t)stream));
+  const int mode = !k ? 1 : std::strcmp(k, "tc") == 0 ? 3 : std::strcmp(k, "line") == 0 ? 4 : std::strcmp(k, "elem") == 0 ? 5 : 1;
+  CUDA_TRY(launch_apply_tile(mode, m->g, x_d, y_d, (cudaStream_t)stream));
   return SEM_OK;
 }
 

@@ -2160,7 +2160,7 @@ cudaError_t launch_stage_cluster_impl(int mixed, int wide, const StageArgs& a, i
 // beyond, one CTA per SM); persistent CTAs (at most the co-resident count) stride over the tiles.
 // The tensor-core FP32 kernel (apply_tc.cuh, fp32 = 3, orders 4..7) takes tiles of 64/Nz − 1
 // elements: with the recomputed left neighbour, 64 element blocks, four block pairs per warp.
-constexpr size_t kTileSmemTarget = 76 * 1024;
+constexpr size_t kTileSmemTarget = 76 * 1024, kTileSmemThird = 75 * 1024 - 64;
 
 template <int P>
 static int tile_grid(const void* fn, size_t smem, int E, int Nx, int slot, cudaError_t* err, int threads = kThreads) {
@@ -2196,10 +2196,39 @@ static int tile_grid(const void* fn, size_t smem, int E, int Nx, int slot, cudaE
 // results no longer fit in a thread's registers), up to four layers.
 constexpr int kElemMaxP = 8;
 
+// Where it serves.  Orders up to 6 from quarters of a tile per SM on; below, tiles of the line passes are smaller and
+// use more of the chip.  Line passes / one element per thread, µs, at the sizes around the line: order 3, one layer
+// 5000 elements 4.3/4.6, 8333 5.0/4.5; order 4 5000 5.0/5.5, 10000 5.8/5.6; order 5 6667 5.1/6.8, 13333 7.6/6.9, two layers 3636
+// 5.4/6.1, 7273 6.1/6.1, 10909 7.5/6.8; order 6 9524 5.9/8.2, 23810 10.3/9.1, two layers 5128 6.1/7.4, 12821 11.2/8.4, four 2667
+// 6.3/7.2, 4000 8.2/7.2.  A mesh of one warp's elements is quicker without the line passes' barriers: 25×1, P = 4 4.6/3.6,
+// 18×3, P = 6 7.4/6.1 (but 13×4 5.0/6.4).  Orders 7 and 8 (188 and 255 registers) run in waves of one or two tiles an SM that last the same
+// however full they are, and win where the waves are nearly full: 26786×1, P = 7 12.6/11.4 (full to 0.69), 44643×1
+// 17.6/20.5 (0.58), 16234×3 18.8/15.2 (0.85), 38095×2 22.2/16.0 (0.99), 23810×2 15.1/16.0 (0.62); 18382×2, P = 8 16.6/14.2 (0.96),
+// 15152×4 24.9/21.5 (0.80), 9470×4 19.0/20.7 (0.50); order 8 with one layer never: 55556×1 24.9/31.3 (0.96).
+template <int P>
+constexpr int elem_quarters(int Nz) {
+  return P <= 2 ? 0 : P <= 4 ? (Nz == 1 ? 2 : 0) : P == 5 ? (Nz == 1 ? 2 : Nz == 2 ? 3 : 0) : 3;
+}
+
+template <int P, int NZ>
+static bool elem_fills_nz(const DevGeom& g) {
+  using L = ElemTile<P, NZ>;
+  if constexpr (P <= 6)
+    return 4LL * g.Nx >= (long long)elem_quarters<P>(NZ) * g.sms * L::E || ((P <= 5 || NZ == 3) && g.Nx < 32);
+  if constexpr (P == 8 && NZ == 1) return false;
+  const long long tiles = (g.Nx + L::E - 1) / L::E, cap = (long long)L::ctas * g.sms, waves = (tiles + cap - 1) / cap;
+  return 100 * tiles >= (P == 7 ? 70 : 77) * waves * cap;
+}
+
 template <int P>
 static bool elem_fills(const DevGeom& g) {
-  const int E = g.Nz == 1 ? ElemTile<P, 1>::E : g.Nz == 2 ? ElemTile<P, 2>::E : g.Nz == 3 ? ElemTile<P, 3>::E : ElemTile<P, 4>::E;
-  return g.Nx >= (P <= 6 ? 76 : 152) * E;
+  switch (g.Nz) {
+    case 1: return elem_fills_nz<P, 1>(g);
+    case 2: return elem_fills_nz<P, 2>(g);
+    case 3: return elem_fills_nz<P, 3>(g);
+    case 4: return elem_fills_nz<P, 4>(g);
+    default: return false;
+  }
 }
 
 template <int P, int NZ>
@@ -2243,10 +2272,7 @@ cudaError_t launch_apply_tile_impl(int fp32, const DevGeom& g, const void* x, vo
     }
   }
   if constexpr (P <= kElemMaxP) {
-    // one element per thread; orders 7 and 8 (255 registers, 2 CTAs an SM) from the size on that gives
-    // every SM a tile: 2.5 M nodes at P = 8 take 23–27 → 17–23 µs, 0.6 M nodes 10–12 → 14–16; order 6 with one
-    // layer (tiles of 127 elements) from half of that: 0.6 M nodes 12.3 → 10.3 µs, 0.16 M 9.3 → 10.2
-    if (fp32 && g.Nz <= 4 && (P <= 5 || (P == 6 && g.Nz > 1) || elem_fills<P>(g))) {
+    if (g.Nz <= 4 && (fp32 == 5 || ((fp32 == 1 || fp32 == 3) && elem_fills<P>(g)))) {   // one element per thread
       const int vec_ok = (reinterpret_cast<uintptr_t>(y) % 16) == 0 ? 1 : 0;
       switch (g.Nz) {
         case 1: return launch_apply_elem<P, 1>(g, xf, yf, bulk_ok, vec_ok, s);
@@ -2261,6 +2287,8 @@ cudaError_t launch_apply_tile_impl(int fp32, const DevGeom& g, const void* x, vo
   const size_t cap = fp32 ? kTileSmemTarget : P <= 8 ? (size_t)112 * 1024 : (size_t)kMaxDynSmem;
   int E = 16;
   while (E > 1 && apply_tile_smem<P>(E, g.nrow, g.Nz, elem) > cap) E >>= 1;
+  if (fp32)   // just above a third of an SM: a narrower tile rather than two CTAs (3049×5, P = 8: 13.4 → 9.6 µs)
+    while (E > 1 && apply_tile_smem<P>(E, g.nrow, g.Nz, elem) > kTileSmemThird) --E;
   const int Et = fp32 ? apply_tile_width(P, g.Nz) : 0;   // a measured FP32 width (autotuner), if set
   if (Et > 0 && apply_tile_smem<P>(Et, g.nrow, g.Nz, elem) <= (size_t)kMaxDynSmem) E = Et;
   const size_t smem = apply_tile_smem<P>(E, g.nrow, g.Nz, elem);
@@ -2271,18 +2299,15 @@ cudaError_t launch_apply_tile_impl(int fp32, const DevGeom& g, const void* x, vo
   const void* fns[5] = {(const void*)k_apply_tile<P, double, 0>, (const void*)k_apply_tile<P, float, 0>,
                         (const void*)k_apply_tile<P, float, 1>, (const void*)k_apply_tile<P, float, 2>,
                         (const void*)k_apply_tile<P, float, 4>};
-  const int grid = tile_grid<P>(fns[k], smem, E, g.Nx, k, &e, fp32 ? kThreads : tile_threads<P, double>());
+  const int threads = fp32 ? kThreads : tile_threads<P, double>();
+  const int grid = tile_grid<P>(fns[k], smem, E, g.Nx, k, &e, threads);
   if (e != cudaSuccess) return e;
-  switch (k) {
-    case 0: k_apply_tile<P, double, 0><<<grid, tile_threads<P, double>(), smem, s>>>(g, static_cast<const double*>(x),
-                                                                   static_cast<double*>(y), E, bulk_ok); break;
-    case 1: k_apply_tile<P, float, 0><<<grid, kThreads, smem, s>>>(g, xf, yf, E, bulk_ok); break;
-    case 2: k_apply_tile<P, float, 1><<<grid, kThreads, smem, s>>>(g, xf, yf, E, bulk_ok); break;
-    case 3: k_apply_tile<P, float, 2><<<grid, kThreads, smem, s>>>(g, xf, yf, E, bulk_ok); break;
-    default: k_apply_tile<P, float, 4><<<grid, kThreads, smem, s>>>(g, xf, yf, E, bulk_ok); break;
-  }
+  DevGeom gg = g;
+  int Ea = E, ba = bulk_ok;
+  void* args[] = {&gg, &x, &y, &Ea, &ba};
+  e = cudaLaunchKernel(fns[k], dim3(grid), dim3(threads), args, smem, s);
   count_launch();
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace semgb
