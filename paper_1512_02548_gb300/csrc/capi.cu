@@ -690,7 +690,7 @@ static int mesh_create_impl(const sem_params* pin, const double* x_edges_h, cons
   const size_t o_S32 = cv.take<float>((size_t)nr * nr), o_ST32 = cv.take<float>((size_t)nr * nr),
                o_lam = cv.take<double>(nr), o_xcol = cv.take<double>(ncol);
   // surface tables
-  const size_t o_tD = cv.take<double>(Q * Q), o_tSX = cv.take<double>(Q * Q), o_tZB = cv.take<double>((size_t)Q * Qf),
+  const size_t o_tSX = cv.take<double>(Q * Q), o_tZB = cv.take<double>((size_t)Q * Qf),
                o_tI = cv.take<double>((size_t)Qf * Q), o_tF = cv.take<double>(Q * Q), o_twr = cv.take<double>((size_t)nrow),
                o_tZ = cv.take<double>((size_t)2 * Pm + 1), o_tse = cv.take<double>(Nx), o_tal = cv.take<double>(N),
                o_tm = cv.take<double>(N), o_tcp = cv.take<double>(N);
@@ -771,7 +771,7 @@ static int mesh_create_impl(const sem_params* pin, const double* x_edges_h, cons
     for (int e = 0; e < Nx; ++e) r2dx[e] = 2.0 / dxe[e];
     up(o_r2dx, r2dx);
   }
-  up(o_tD, L.D); up(o_tSX, ct->SX); up(o_tZB, ct->ZB); up(o_tI, I); up(o_tF, F); up(o_twr, wrow);
+  up(o_tSX, ct->SX); up(o_tZB, ct->ZB); up(o_tI, I); up(o_tF, F); up(o_twr, wrow);
   up(o_tZ, Z); up(o_tse, se); up(o_tal, th_al); up(o_tm, th_m); up(o_tcp, th_cp);
   up(o_lam, lam);
   {
@@ -850,8 +850,8 @@ static int mesh_create_impl(const sem_params* pin, const double* x_edges_h, cons
 
   SurfTables& t = m->st;
   t.P = P; t.Pf = p.Pf; t.Nx = Nx; t.Nz = Nz; t.ncol = ncol; t.nrow = nrow; t.periodic = g.periodic; t.g = p.g;
-  t.D = D_(o_tD); t.SX = D_(o_tSX); t.ZB = D_(o_tZB); t.I = D_(o_tI); t.F = D_(o_tF); t.wrow = D_(o_twr);
-  t.Z = D_(o_tZ); t.se = D_(o_tse); t.r2dx = g.r2dx; t.dsl = g.dsl; t.h = g.h;
+  t.SX = D_(o_tSX); t.ZB = D_(o_tZB); t.I = D_(o_tI); t.F = D_(o_tF); t.wrow = D_(o_twr);
+  t.Z = D_(o_tZ); t.se = D_(o_tse); t.r2dx = g.r2dx; t.h = g.h;
   t.th_al = D_(o_tal); t.th_m = D_(o_tm); t.th_cp = D_(o_tcp); t.win = ct->win; t.nif = N; t.filter_on = (p.filter_ic >= 0 && p.filter_ic < P) ? 1 : 0;
   t.xcol = D_(o_xcol); t.x0 = x_edges_h[0]; t.x1 = x_edges_h[Nx];
   t.relax_left = p.relax_left; t.relax_right = p.relax_right; t.ncomp = 0; t.wave = D_(o_wave);

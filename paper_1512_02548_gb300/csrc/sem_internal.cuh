@@ -161,7 +161,6 @@ struct PcgArgs {
 struct SurfTables {
   int P, Pf, Nx, Nz, ncol, nrow, periodic;
   double g;
-  const double* D;        // (P+1)²  differentiation on the GLL nodes
   const double* SX;       // (P+1)²  M·D, rows condensed (surface_device.cuh)
   const double* ZB;       // (P+1)×(Pf+1)  Iᵀ M_f (over-integration projection), rows condensed
   const double* I;        // (Pf+1)×(P+1)  interpolation to the fine nodes
@@ -170,7 +169,6 @@ struct SurfTables {
   const double* Z;        // 2×(P−1) M_bi M_ii⁻¹
   const double* se;       // [Nx] Δx_e / 2
   const double* r2dx;     // [Nx] 2/Δx_e
-  const double* dsl;      // [Nz]
   const double* h;        // [ncol]
   const double* th_al;    // interface system of M': −e_{j−1} m_j       [N]
   const double* th_m;     // 1/pivot m_j (cyclic factors when periodic) [N]
