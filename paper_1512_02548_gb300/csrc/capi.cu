@@ -1303,8 +1303,12 @@ double estimate_cooperative(const sem_batch* b) {
 // up, and the launches of all groups run at the same time on streams of their own.  The largest
 // cluster is the one of 4, 8 and 16 CTAs (at most the tuned maximum) with the best estimate: few tanks
 // are bound by the longest team, many by the CTA slots, where every further CTA costs its chain.
-// Members are grouped by (order, precision, c), the largest first within a launch.  Returns
-// false (and builds nothing) when some group's cluster does not fit on the device; *estimate: its stage time.
+// Members are grouped by (order, precision, c), the largest first within a launch.  Where some group's cluster
+// does not fit on the device, the next best of the three is taken.  Returns false (and builds nothing) when none
+// fits; *estimate: its stage time.
+bool build_clusters(sem_batch* b, sem_mesh* const* meshes, int count, const std::vector<double>& w, double per_cta,
+                    int cap);
+
 bool plan_clusters(sem_batch* b, sem_mesh* const* meshes, int count, int sms, double* estimate) {
   std::vector<double> w(count);
   double total = 0.0;
@@ -1315,12 +1319,20 @@ bool plan_clusters(sem_batch* b, sem_mesh* const* meshes, int count, int sms, do
   const sem_batch_tuning tune = batch_tuning();
   const double slots = 2.0 * sms;
   const double per_cta = tune.cluster_share * total / slots;
-  int cap = std::min(4, tune.max_cluster);
-  *estimate = estimate_clusters(meshes, w, per_cta, cap, slots);
-  for (int c = 8; c <= tune.max_cluster; c *= 2) {
-    const double e = estimate_clusters(meshes, w, per_cta, c, slots);
-    if (e < *estimate) { *estimate = e; cap = c; }
-  }
+  std::vector<std::pair<double, int>> caps;    // (estimate, cap), the best first
+  for (int c = std::min(4, tune.max_cluster); c <= tune.max_cluster; c *= 2)
+    caps.emplace_back(estimate_clusters(meshes, w, per_cta, c, slots), c);
+  std::sort(caps.begin(), caps.end());
+  for (const auto& c : caps)
+    if (build_clusters(b, meshes, count, w, per_cta, c.second)) {
+      *estimate = c.first;
+      return true;
+    }
+  return false;
+}
+
+bool build_clusters(sem_batch* b, sem_mesh* const* meshes, int count, const std::vector<double>& w, double per_cta,
+                    int cap) {
   std::vector<std::pair<std::array<int, 3>, std::vector<int>>> groups;
   for (int i = 0; i < count; ++i) {
     const int c = cluster_size(meshes[i], w[i], per_cta, cap);
