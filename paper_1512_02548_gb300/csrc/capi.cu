@@ -211,6 +211,12 @@ struct sem_batch {
   std::vector<int> codes;            // per-instance error code of the last step or solve
   std::vector<BatchLaunch> launches;     // cooperative plan: one launch per RK stage and group
   std::vector<BatchLaunch> cl_launches;  // cluster plan: launches on streams of their own (empty: none)
+  // the Laplace solves' plan, made by the first of them: −1 not made, 0 cooperative, 1 the steps' clusters, 2 cl_solve
+  int solve_plan = -1;
+  std::vector<BatchLaunch> cl_solve;
+  unsigned char* solve_pool = nullptr;
+  sem_batch_tuning tune{};
+  int force = -1;                        // plan asked for: −1 the faster by estimate, 0 cooperative, 1 clusters
   cudaEvent_t fork = nullptr;
   int device = 0;
   unsigned char* pool = nullptr;
@@ -1306,17 +1312,17 @@ double estimate_cooperative(const sem_batch* b) {
 // Members are grouped by (order, precision, c), the largest first within a launch.  Where some group's cluster
 // does not fit on the device, the next best of the three is taken.  Returns false (and builds nothing) when none
 // fits; *estimate: its stage time.
-bool build_clusters(sem_batch* b, sem_mesh* const* meshes, int count, const std::vector<double>& w, double per_cta,
-                    int cap);
+bool build_clusters(std::vector<BatchLaunch>* plan, sem_mesh* const* meshes, int count, const std::vector<double>& w,
+                    double per_cta, int cap);
 
-bool plan_clusters(sem_batch* b, sem_mesh* const* meshes, int count, int sms, double* estimate) {
+bool plan_clusters(std::vector<BatchLaunch>* plan, sem_mesh* const* meshes, int count, int sms,
+                   const sem_batch_tuning& tune, double* estimate) {
   std::vector<double> w(count);
   double total = 0.0;
   for (int i = 0; i < count; ++i) {
     w[i] = member_work(meshes[i]);
     total += w[i];
   }
-  const sem_batch_tuning tune = batch_tuning();
   const double slots = 2.0 * sms;
   const double per_cta = tune.cluster_share * total / slots;
   std::vector<std::pair<double, int>> caps;    // (estimate, cap), the best first
@@ -1324,15 +1330,15 @@ bool plan_clusters(sem_batch* b, sem_mesh* const* meshes, int count, int sms, do
     caps.emplace_back(estimate_clusters(meshes, w, per_cta, c, slots), c);
   std::sort(caps.begin(), caps.end());
   for (const auto& c : caps)
-    if (build_clusters(b, meshes, count, w, per_cta, c.second)) {
+    if (build_clusters(plan, meshes, count, w, per_cta, c.second)) {
       *estimate = c.first;
       return true;
     }
   return false;
 }
 
-bool build_clusters(sem_batch* b, sem_mesh* const* meshes, int count, const std::vector<double>& w, double per_cta,
-                    int cap) {
+bool build_clusters(std::vector<BatchLaunch>* plan, sem_mesh* const* meshes, int count, const std::vector<double>& w,
+                    double per_cta, int cap) {
   std::vector<std::pair<std::array<int, 3>, std::vector<int>>> groups;
   for (int i = 0; i < count; ++i) {
     const int c = cluster_size(meshes[i], w[i], per_cta, cap);
@@ -1372,7 +1378,7 @@ bool build_clusters(sem_batch* b, sem_mesh* const* meshes, int count, const std:
     L.smem = smem_l;
     out.push_back(std::move(L));
   }
-  b->cl_launches = std::move(out);
+  *plan = std::move(out);
   return true;
 }
 
@@ -1406,16 +1412,16 @@ void release_plan(std::vector<BatchLaunch>& plan, int dev) {
 }
 
 
-// A plan's device arrays (descriptors, CTA map, barrier words, gathered status) from the pool.
-int carve_plan(sem_batch* b, std::vector<BatchLaunch>& plan, size_t& off) {
+// A plan's device arrays (descriptors, CTA map, barrier words, gathered status) from `pool`.
+int carve_plan(int dev, unsigned char* pool, std::vector<BatchLaunch>& plan, size_t& off) {
   for (auto& L : plan) {
-    L.inst_d = reinterpret_cast<Instance*>(b->pool + off);
+    L.inst_d = reinterpret_cast<Instance*>(pool + off);
     off += (sizeof(Instance) * L.members.size() + 255) & ~size_t(255);
-    L.cta_d = reinterpret_cast<int*>(b->pool + off);
+    L.cta_d = reinterpret_cast<int*>(pool + off);
     off += (sizeof(int) * (size_t)L.grid + 255) & ~size_t(255);
-    L.bars_d = reinterpret_cast<unsigned int*>(b->pool + off);
+    L.bars_d = reinterpret_cast<unsigned int*>(pool + off);
     off += (sizeof(unsigned) * 2 * L.members.size() + 255) & ~size_t(255);
-    L.status_d = reinterpret_cast<int*>(b->pool + off);
+    L.status_d = reinterpret_cast<int*>(pool + off);
     off += (sizeof(int) * L.members.size() + 255) & ~size_t(255);
     std::vector<int> map(L.grid);
     for (size_t k = 0; k < L.members.size(); ++k)
@@ -1423,7 +1429,7 @@ int carve_plan(sem_batch* b, std::vector<BatchLaunch>& plan, size_t& off) {
     CUDA_TRY(cudaMemcpy(L.cta_d, map.data(), sizeof(int) * L.grid, cudaMemcpyHostToDevice));
     L.inst_h.resize(L.members.size());
     L.status_h.resize(L.members.size());
-    if (L.csize > 0) CUDA_TRY(take_stream(b->device, &L.stream, &L.done));
+    if (L.csize > 0) CUDA_TRY(take_stream(dev, &L.stream, &L.done));
   }
   return SEM_OK;
 }
@@ -1436,6 +1442,48 @@ size_t plan_bytes(const std::vector<BatchLaunch>& plan) {
              ((sizeof(unsigned) * 2 * L.members.size() + 255) & ~size_t(255)) +
              ((sizeof(int) * L.members.size() + 255) & ~size_t(255));
   return total;
+}
+
+// The plan of the Laplace solves of a batch whose steps run in clusters.  A solve from a caller's start takes several
+// times a stage's iterations between the same fixed phases, so a CTA's chain weighs less and larger teams pay: the
+// cluster plan at half the steps' share, or the cooperative one where that is estimated faster.  Solves from zero, ms, on
+// the steps' plan / on this one: 512 tanks 6.25 / 5.53 FP64 and 5.48 / 4.93 mixed, 200 3.25 / 2.85, 100 2.28 / 1.74.
+// (Steps at half the share: 512 tanks 9.45 → 9.65 ms.)  Without memory for it the steps' plan serves.
+void plan_solves(sem_batch* b) {
+  b->solve_plan = 1;
+  int sms = 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device) != cudaSuccess) return;
+  sem_batch_tuning tune = b->tune;
+  tune.cluster_share *= 0.5;
+  std::vector<BatchLaunch> plan;
+  double est = 0.0;
+  const int count = (int)b->meshes.size();
+  if (!plan_clusters(&plan, b->meshes.data(), count, sms, tune, &est)) return;
+  if (b->force < 0 && est > estimate_cooperative(b)) {
+    b->solve_plan = 0;
+    return;
+  }
+  std::vector<int> size(count);
+  for (const auto& L : b->cl_launches)
+    for (int i : L.members) size[i] = L.csize;
+  bool same = true;
+  for (const auto& L : plan)
+    for (int i : L.members) same = same && size[i] == L.csize;
+  if (same) return;
+  size_t off = 0;
+  if (dev_alloc(b->device, plan_bytes(plan) + 256, reinterpret_cast<void**>(&b->solve_pool)) != cudaSuccess) {
+    cudaGetLastError();
+    b->solve_pool = nullptr;
+    return;
+  }
+  if (carve_plan(b->device, b->solve_pool, plan, off) != SEM_OK) {
+    release_plan(plan, b->device);
+    dev_free(b->device, b->solve_pool);
+    b->solve_pool = nullptr;
+    return;
+  }
+  b->cl_solve = std::move(plan);
+  b->solve_plan = 2;
 }
 
 }  // namespace
@@ -1467,9 +1515,11 @@ int sem_batch_create(sem_mesh* const* meshes, int count, sem_batch** out) {
   // when a few large members would need more CTAs than a cluster holds); SEM_BATCH_CLUSTER=0 or 1
   // forces either plan.
   const char* cenv = std::getenv("SEM_BATCH_CLUSTER");
-  const int force = cenv ? (std::atoi(cenv) != 0 ? 1 : 0) : batch_tuning().plan;
+  b->tune = batch_tuning();
+  const int force = b->force = cenv ? (std::atoi(cenv) != 0 ? 1 : 0) : b->tune.plan;
   double est = 0.0;
-  if (force != 0 && plan_clusters(b, meshes, count, sms, &est) && force < 0 && est > estimate_cooperative(b))
+  if (force != 0 && plan_clusters(&b->cl_launches, meshes, count, sms, b->tune, &est) && force < 0 &&
+      est > estimate_cooperative(b))
     b->cl_launches.clear();
   for (int i = 0; i < count; ++i) {
     b->off.push_back(b->ncol_total);
@@ -1481,8 +1531,8 @@ int sem_batch_create(sem_mesh* const* meshes, int count, sem_batch** out) {
   if (ae != cudaSuccess) { delete b; return fail(SEM_ERR_OOM, std::string("cudaMalloc: ") + cudaGetErrorString(ae)); }
   b->state = reinterpret_cast<double*>(b->pool);
   size_t off = state_bytes;
-  rc = carve_plan(b, b->launches, off);
-  if (!rc) rc = carve_plan(b, b->cl_launches, off);
+  rc = carve_plan(dev, b->pool, b->launches, off);
+  if (!rc) rc = carve_plan(dev, b->pool, b->cl_launches, off);
   if (!rc && !b->cl_launches.empty() && cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) != cudaSuccess)
     rc = fail(SEM_ERR_CUDA, "event creation failed");
   if (rc) {
@@ -1500,9 +1550,11 @@ void sem_batch_destroy(sem_batch* b) {
   DeviceGuard dg(b->device);
   cudaDeviceSynchronize();   // no work of this batch may still run when its memory is reused
   release_plan(b->cl_launches, b->device);
+  release_plan(b->cl_solve, b->device);
   if (b->fork) cudaEventDestroy(b->fork);
   for (auto& pr : b->events) { cudaEventDestroy(pr.first); cudaEventDestroy(pr.second); }
   for (cudaEvent_t e : b->spare) cudaEventDestroy(e);
+  if (b->solve_pool) dev_free(b->device, b->solve_pool);
   dev_free(b->device, b->pool);
   delete b;
 }
@@ -1573,20 +1625,20 @@ cudaError_t batch_launch(sem_batch* b, const BatchLaunch& L, const StageArgs& a,
   return cudaSuccess;
 }
 
-// The cluster plan: each group's stage launches in order on the group's own stream, the streams
+// A cluster plan: each group's stage launches in order on the group's own stream, the streams
 // forked from and joined back to s.  stage 0: the Laplace solve alone; else nsteps RK4 steps.
-cudaError_t run_clusters(sem_batch* b, int stage, int nsteps, cudaStream_t s) {
+cudaError_t run_clusters(sem_batch* b, std::vector<BatchLaunch>& plan, int stage, int nsteps, cudaStream_t s) {
   cudaError_t e;
   if ((e = cudaEventRecord(b->fork, s)) != cudaSuccess) return e;
-  for (auto& L : b->cl_launches)
+  for (auto& L : plan)
     if ((e = cudaStreamWaitEvent(L.stream, b->fork, 0)) != cudaSuccess) return e;
   for (int step = 0; step < (stage == 0 ? 1 : nsteps); ++step)
     for (int st = (stage == 0 ? 0 : 1); st <= (stage == 0 ? 0 : 4); ++st)
-      for (auto& L : b->cl_launches) {
+      for (auto& L : plan) {
         const StageArgs a{L.inst_d, L.cta_d, nullptr, st, step, 1, {}};
         if ((e = batch_launch(b, L, a, L.stream)) != cudaSuccess) return e;
       }
-  for (auto& L : b->cl_launches) {
+  for (auto& L : plan) {
     if ((e = cudaEventRecord(L.done, L.stream)) != cudaSuccess) return e;
     if ((e = cudaStreamWaitEvent(s, L.done, 0)) != cudaSuccess) return e;
   }
@@ -1616,7 +1668,7 @@ int sem_batch_rk4_step(sem_batch* b, double* const* eta_d, double* const* phis_d
                              cudaMemcpyHostToDevice, s));
   }
   if (cl) {
-    if (nsteps > 0) CUDA_TRY(run_clusters(b, 1, nsteps, s));
+    if (nsteps > 0) CUDA_TRY(run_clusters(b, plan, 1, nsteps, s));
   } else {
     for (int step = 0; step < nsteps; ++step)
       for (int stage = 1; stage <= 4; ++stage)
@@ -1642,8 +1694,10 @@ int sem_batch_laplace_solve(sem_batch* b, const double* const* eta_d, const doub
     if (!eta_d[i] || !phis_d[i] || !Phi_d[i]) return fail(SEM_ERR_INVALID_ARG, "bad instance state");
   DeviceGuard dg(b->device);
   cudaStream_t s = (cudaStream_t)stream;
-  const bool cl = use_clusters(b);
-  auto& plan = cl ? b->cl_launches : b->launches;
+  bool cl = use_clusters(b);
+  if (cl && b->solve_plan < 0) plan_solves(b);
+  cl = cl && b->solve_plan != 0;
+  auto& plan = !cl ? b->launches : b->solve_plan == 2 ? b->cl_solve : b->cl_launches;
   for (auto& L : plan) {
     for (size_t k = 0; k < L.members.size(); ++k) {
       const int i = L.members[k];
@@ -1655,7 +1709,7 @@ int sem_batch_laplace_solve(sem_batch* b, const double* const* eta_d, const doub
                              cudaMemcpyHostToDevice, s));
   }
   if (cl) {
-    CUDA_TRY(run_clusters(b, 0, 0, s));
+    CUDA_TRY(run_clusters(b, plan, 0, 0, s));
   } else {
     for (auto& L : plan) {
       CUDA_TRY(cudaMemsetAsync(L.bars_d, 0, 2 * sizeof(unsigned int) * L.members.size(), s));
