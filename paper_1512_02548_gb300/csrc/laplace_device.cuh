@@ -2160,7 +2160,7 @@ cudaError_t launch_stage_cluster_impl(int mixed, int wide, const StageArgs& a, i
 // beyond, one CTA per SM); persistent CTAs (at most the co-resident count) stride over the tiles.
 // The tensor-core FP32 kernel (apply_tc.cuh, fp32 = 3, orders 4..7) takes tiles of 64/Nz − 1
 // elements: with the recomputed left neighbour, 64 element blocks, four block pairs per warp.
-constexpr size_t kTileSmemTarget = 76 * 1024, kTileSmemThird = 75 * 1024 - 64;
+constexpr size_t kTileSmemTarget = 76 * 1024;
 
 template <int P>
 static int tile_grid(const void* fn, size_t smem, int E, int Nx, int slot, cudaError_t* err, int threads = kThreads) {
@@ -2287,8 +2287,11 @@ cudaError_t launch_apply_tile_impl(int fp32, const DevGeom& g, const void* x, vo
   const size_t cap = fp32 ? kTileSmemTarget : P <= 8 ? (size_t)112 * 1024 : (size_t)kMaxDynSmem;
   int E = 16;
   while (E > 1 && apply_tile_smem<P>(E, g.nrow, g.Nz, elem) > cap) E >>= 1;
-  if (fp32)   // just above a third of an SM: a narrower tile rather than two CTAs (3049×5, P = 8: 13.4 → 9.6 µs)
-    while (E > 1 && apply_tile_smem<P>(E, g.nrow, g.Nz, elem) > kTileSmemThird) --E;
+  // one element less where that lets an SM hold one CTA more (3049×5, P = 8: 13.4 → 9.6 µs, 53333×8, P = 3: 41 → 37)
+  for (int n = 3; fp32 && n <= 6; ++n) {
+    const size_t share = (size_t)228 * 1024 / n - 1024 - 64;
+    if (E >= 7 && apply_tile_smem<P>(E, g.nrow, g.Nz, elem) > share && apply_tile_smem<P>(E - 1, g.nrow, g.Nz, elem) <= share) --E;
+  }
   const int Et = fp32 ? apply_tile_width(P, g.Nz) : 0;   // a measured FP32 width (autotuner), if set
   if (Et > 0 && apply_tile_smem<P>(Et, g.nrow, g.Nz, elem) <= (size_t)kMaxDynSmem) E = Et;
   const size_t smem = apply_tile_smem<P>(E, g.nrow, g.Nz, elem);
