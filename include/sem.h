@@ -110,7 +110,7 @@ typedef struct sem_info {
   int ncol, nrow;
   int n_elements;      /* Nx·Nz                               */
   int P, Pf, Nx, Nz, periodic, precision;
-  int grid_ctas;       /* CTAs of the persistent Krylov kernel */
+  int grid_ctas;       /* CTAs of the stand-alone solve's launch */
   int stage_ctas;      /* CTAs of the fused RK stage launch    */
   int64_t device_bytes;/* device memory owned by the mesh      */
 } sem_info;

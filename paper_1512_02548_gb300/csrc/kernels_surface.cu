@@ -25,9 +25,9 @@ __host__ __device__ static inline int rec_blocks(int Nx) { return (Nx + kRecElem
 
 // Gradient recovery, latency bound, in one launch of two kinds of blocks.  The first nrec = Nx/16 take S_x of η
 // and φ̃ (boundary rows for the whole window, kept in shared memory), the interface solves and their
-// columns of ∂xη and ∂xφ̃; the others w̃ of 16 columns each.  In the blocks of the solves, w̃ had made few
-// blocks of high order work through hundreds of columns (26×8, P = 12: 54 µs; the three launches before
-// them 21).
+// columns of ∂xη and ∂xφ̃; the others w̃ of 16 columns each: in the blocks of the solves it had made few
+// blocks of high order work through hundreds of columns.  26×8, P = 12, called from the host: three launches
+// 21 µs, w̃ in the solves' blocks 54, now 10; in a graph 16.6 and 11.3, 687×8 166 and 12.8.
 __global__ void __launch_bounds__(kRecThreads) k_recover(SurfTables t, const double* __restrict__ Phi,
                                                          const double* __restrict__ eta,
                                                          const double* __restrict__ phis, double* __restrict__ w,

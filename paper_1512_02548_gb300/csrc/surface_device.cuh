@@ -71,14 +71,15 @@ __device__ __forceinline__ void sx_item(const SurfTables& t, const double* __res
 
 // Interface unknowns lo, lo+1, …, lo+cnt−1 (cyclic when periodic) of the condensed M' system, by one
 // warp, from the right-hand side gfun(j), 0 ≤ j < N; store(i, u) receives unknown lo + i.
-// The system's LDLᵀ factors decay: with the multipliers l_j = e_j/p_j, |l_j| ≤ |S01|/S00 = 1/(P+1) for
-// any element widths, so the recurrences
+// The system's LDLᵀ factors decay, so the recurrences
 //     y_j = g_j m_j − (e_{j−1} m_j) y_{j−1},        u_j = y_j − l_j u_{j+1}
 // started t.win interfaces away from the first unknown wanted (and from zero) agree with the whole
-// chain's to (P+1)^−win < 1e-18.  Every CTA therefore solves for its own elements alone, without
-// waiting for a solve of the whole chain elsewhere: an RK stage has four team barriers fewer and no
-// 2049-unknown solve on two CTAs while the others wait (step on the 2048×2 shoal 1849 → 1729 µs, on 64×4
-// 721 → 700 µs, 512 uneven tanks 12.52 → 12.17 ms).  The periodic chain uses the cyclic factors (the fixed point of the pivot recurrence around the ring), no closure.
+// chain's.  For any element widths |l_j| = |e_j|/p_j ≤ |S01|/S00 = 1/(P+1), which makes (P+1)^−win < 1e-18
+// for the second; the first has p_j ≥ Δx_{j−1}/2 (S11 − |S01|/(P+1)), so |e_{j−1}| m_j ≤ (P+1)/((P+1)² − 1): below 1e-18
+// where the widths vary little, at most 7e-17 (order 2, every element far narrower than the one before it).
+// Every CTA therefore solves for its own elements alone, without waiting for a solve of the whole chain
+// elsewhere: an RK stage has four team barriers fewer and no 2049-unknown solve on two CTAs while the others wait.
+// The periodic chain uses the cyclic factors (the fixed point of the pivot recurrence around the ring), no closure.
 // Lanes hold chunks of c ≤ kWinRegs positions of the window; the composed affine maps are scanned
 // over as many lanes as cover t.win positions.
 constexpr int kWinRegs = 6;
