@@ -1412,21 +1412,27 @@ void release_plan(std::vector<BatchLaunch>& plan, int dev) {
 }
 
 
-// A plan's device arrays (descriptors, CTA map, barrier words, gathered status) from `pool`.
+// A plan's device arrays (CTA maps, descriptors, barrier words, gathered status) from `pool`; the maps of all
+// its launches lie together and go up in one copy (a copy each had cost a server's tick 10 µs a launch).
 int carve_plan(int dev, unsigned char* pool, std::vector<BatchLaunch>& plan, size_t& off) {
+  const size_t first = off;
+  std::vector<int> maps;
+  for (auto& L : plan) {
+    L.cta_d = reinterpret_cast<int*>(pool + off);
+    off += (sizeof(int) * (size_t)L.grid + 255) & ~size_t(255);
+    const size_t at = ((unsigned char*)L.cta_d - (pool + first)) / sizeof(int);
+    maps.resize((off - first) / sizeof(int), 0);
+    for (size_t k = 0; k < L.members.size(); ++k)
+      for (int c = 0; c < L.nteam[k]; ++c) maps[at + L.team0[k] + c] = (int)k;
+  }
+  if (!maps.empty()) CUDA_TRY(cudaMemcpy(pool + first, maps.data(), sizeof(int) * maps.size(), cudaMemcpyHostToDevice));
   for (auto& L : plan) {
     L.inst_d = reinterpret_cast<Instance*>(pool + off);
     off += (sizeof(Instance) * L.members.size() + 255) & ~size_t(255);
-    L.cta_d = reinterpret_cast<int*>(pool + off);
-    off += (sizeof(int) * (size_t)L.grid + 255) & ~size_t(255);
     L.bars_d = reinterpret_cast<unsigned int*>(pool + off);
     off += (sizeof(unsigned) * 2 * L.members.size() + 255) & ~size_t(255);
     L.status_d = reinterpret_cast<int*>(pool + off);
     off += (sizeof(int) * L.members.size() + 255) & ~size_t(255);
-    std::vector<int> map(L.grid);
-    for (size_t k = 0; k < L.members.size(); ++k)
-      for (int c = 0; c < L.nteam[k]; ++c) map[L.team0[k] + c] = (int)k;
-    CUDA_TRY(cudaMemcpy(L.cta_d, map.data(), sizeof(int) * L.grid, cudaMemcpyHostToDevice));
     L.inst_h.resize(L.members.size());
     L.status_h.resize(L.members.size());
     if (L.csize > 0) CUDA_TRY(take_stream(dev, &L.stream, &L.done));
