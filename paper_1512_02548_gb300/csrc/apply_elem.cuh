@@ -11,8 +11,8 @@ namespace semgb {
 // lines between its three passes through shared memory.  Here a thread loads the (P+1)² values of its
 // element once, keeps every intermediate in registers, and exchanges only the top row and the right
 // column with its neighbours: about 43 FP32 operations per node.  What bounds it is the latency of a thread's long
-// chains at 12 warps an SM (6 at order 8, 1 or 2 CTAs by registers and shared memory), 58% of the issue slots used.
-// 65536×4, P = 6: 63.5 → 30.5 µs (2.6 TB/s of x and y); 8 M nodes of P = 3..8: 51–138 → 25–62 µs.
+// chains at 12 warps an SM (6 at order 8, 1 or 2 CTAs by registers and shared memory), 60% of the issue slots used.
+// 65536×4, P = 6: 63.5 → 31.0 µs (2.5 TB/s of x and y); 8 M nodes of P = 3..8: 51–138 → 25–62 µs.
 // A warp holds 32 consecutive elements of one layer; a CTA holds all layers of 32·G elements, the first
 // of which is the element left of its tile, recomputed for the tile's first column.  x is staged by bulk
 // copies, double-buffered as in k_apply_tile; y goes through the same buffer and leaves in contiguous
